@@ -232,10 +232,16 @@ dmc_decode_kernel(const DecodeArgs a) {
   // ---------------------------------------------------------------- prologue
   scan_units(U, misc, ctl, L.lengths + (size_t)layer * 2 * L.NH, L.NH, NVH, Gv);
   const long long Utot = U[NVH];
-  const int NW = gridDim.x * NWARP;
-  const int wid = blockIdx.x * NWARP + warp;
-  const int u0 = (int)range_start(wid, Utot, NW);
-  const int u1 = (int)range_start(wid + 1, Utot, NW);
+  // A layer with fewer units than warps gives the first Utot workers one unit
+  // each, spread over the blocks so that every SM takes part. Such a launch is
+  // all latency: cutting the list over every warp left empty ranges between
+  // the parts, which each finish and merge had to step over (7B shape, batch 1,
+  // ~550 units on 1824 warps: 45.2 us per launch, 13.1 with one unit each).
+  const bool few = Utot < (long long)gridDim.x * NWARP;
+  const int NW = few ? (int)Utot : (int)gridDim.x * NWARP;
+  const int wid = few ? warp * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * NWARP + warp;
+  const int u0 = wid < NW ? (int)range_start(wid, Utot, NW) : 0;
+  const int u1 = wid < NW ? (int)range_start(wid + 1, Utot, NW) : 0;
   const int grp = lane >> 3, l8 = lane & 7;
   const uint32_t ring_s = smem_u32(ring);
 
@@ -652,55 +658,21 @@ dmc_decode_kernel(const DecodeArgs a) {
           __syncwarp();
           const int wf = worker_of_unit(hu0, Utot, NW);
           const int wl = worker_of_unit(hend - 1, Utot, NW);
-          // With at least one unit per worker every worker in [wf, wl] holds
-          // part of the head; otherwise some ranges in it are empty.
-          const bool dense = Utot >= NW;
           int last = 0;
           if (lane == 0) {
-            int ncontrib = wl - wf + 1;
-            if (!dense) {
-              ncontrib = 0;
-              for (int cw = wf; cw <= wl; ++cw)
-                ncontrib += range_start(cw, Utot, NW) < range_start(cw + 1, Utot, NW);
-            }
+            // every worker in [wf, wl] holds part of the head
             int* cnt = L.counters + (size_t)layer * L.NH * L.G + vh;
             const int old = atomicAdd(cnt, 1);
-            last = (old == ncontrib - 1);
+            last = (old == wl - wf);
             if (last) *cnt = 0;
           }
           last = __shfl_sync(0xffffffffu, last, 0);
           if (last) {
             __threadfence();  // every contributor's partial is visible to this lane
-            if (dense) {
-              // worker wf + i wrote state 2 (wf + i) + 1 if the head starts
-              // inside its range (only possible for i = 0), else 2 (wf + i)
-              const int first_off = (hu0 > range_start(wf, Utot, NW)) ? 1 : 0;
-              combine_partials<T, D>(partials, wf, first_off, wl - wf + 1, lane, orow);
-            } else {
-              // fewer units than workers (tiny caches): one unit per non-empty
-              // range, so each contributor wrote state 2 cw of its range
-              float Mc = -INFINITY, Lc = 0.f;
-              for (int cw = wf; cw <= wl; ++cw) {
-                if (range_start(cw, Utot, NW) == range_start(cw + 1, Utot, NW)) continue;
-                Mc = fmaxf(Mc, __ldcg(partials + (size_t)(2 * cw) * PSTRIDE));
-              }
-              constexpr int DPL = D / 32;  // output dims per lane
-              float Oc[DPL];
-#pragma unroll
-              for (int i = 0; i < DPL; ++i) Oc[i] = 0.f;
-              for (int cw = wf; cw <= wl; ++cw) {
-                if (range_start(cw, Utot, NW) == range_start(cw + 1, Utot, NW)) continue;
-                const float* cp = partials + (size_t)(2 * cw) * PSTRIDE;
-                const float mc = __ldcg(cp);
-                const float cwt = (mc == -INFINITY) ? 0.f : exp2f(mc - Mc);
-                Lc = fmaf(__ldcg(cp + 1), cwt, Lc);
-#pragma unroll
-                for (int i = 0; i < DPL; ++i) Oc[i] = fmaf(__ldcg(cp + 4 + lane * DPL + i), cwt, Oc[i]);
-              }
-              const float inv = 1.f / Lc;
-#pragma unroll
-              for (int i = 0; i < DPL; ++i) orow[lane * DPL + i] = Elt<T>::from_f(Oc[i] * inv);
-            }
+            // worker wf + i wrote state 2 (wf + i) + 1 if the head starts
+            // inside its range (only possible for i = 0), else 2 (wf + i)
+            const int first_off = (hu0 > range_start(wf, Utot, NW)) ? 1 : 0;
+            combine_partials<T, D>(partials, wf, first_off, wl - wf + 1, lane, orow);
           }
         }
         m = -INFINITY;
