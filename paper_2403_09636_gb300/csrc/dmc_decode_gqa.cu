@@ -81,6 +81,74 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// Workers of a layer of U units over nh heads, on a grid of `warps` warps. A
+// worker streams a page unit in about kUnitCost times what the merge of a split
+// head spends per contributor, so a head of n units is done soonest with about
+// sqrt(kUnitCost n) contributors; more units than that per worker are only taken
+// when the grid has no more warps. Measured for 64 query heads over 8 KV heads,
+// 2048 tokens at 2x, us per launch at batch 1 / 4: 80.6 / 74.0 with every warp a
+// worker and a serial merge; with the merge below and kUnitCost 1, 3, 8: 20.1 /
+// 23.4, 20.1 / 24.4, 23.8 / 31.3.
+constexpr float kUnitCost = 2.f;
+__device__ __forceinline__ int gqa_workers(long long U, int nh, int warps) {
+  const float per_head = (float)U / (float)nh;
+  const float per_worker = fmaxf(1.f, sqrtf(per_head * (1.f / kUnitCost)));
+  const int want = max(1, (int)((float)U / per_worker));
+  return (int)min((long long)min(want, warps), U);
+}
+
+// The last contributor of a split head merges the nc workers' states (wf ..
+// wf + nc - 1, in worker order) and writes the group's output rows. Lane (g =
+// lane / 4, t = lane % 4) sums query g over the dims 8 i + 2 t, + 1 (i = 0 ..
+// D / 8 - 1: four lanes read 32 bytes of a row), two contributors' loads in
+// flight (four in flight: 18.9 us instead of 20.1 at batch 1, but the registers
+// they take spill in the caller, 99.1 against 94.4 us per 70B batch-64 launch).
+template <int D>
+__device__ __noinline__ void combine_gqa(const float* partials, int wf, int first_off, int nc, int G,
+                                         int lane, __nv_bfloat16* ob) {
+  constexpr int NB = 2, V2 = D / 8;
+  const int g = lane >> 2, t = lane & 3;
+  const bool on = g < G;
+  const size_t PS = (size_t)G * (D + 2);
+  const float* row = partials + (size_t)(on ? g : 0) * (D + 2);
+  auto state = [&](int i) { return row + (size_t)(2 * (wf + i) + (i == 0 ? first_off : 0)) * PS; };
+  float Mc = -INFINITY;
+#pragma unroll 4
+  for (int i = t; i < nc; i += 4) Mc = fmaxf(Mc, __ldcg(state(i)));
+  Mc = fmaxf(Mc, __shfl_xor_sync(0xffffffffu, Mc, 1));
+  Mc = fmaxf(Mc, __shfl_xor_sync(0xffffffffu, Mc, 2));
+  float Lc = 0.f;
+  float2 o[V2];
+#pragma unroll
+  for (int i = 0; i < V2; ++i) o[i] = make_float2(0.f, 0.f);
+  for (int i0 = 0; i0 < nc; i0 += NB) {
+    float2 ml[NB], v[NB][V2];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const bool in = i0 + b < nc;
+      const float2* p = reinterpret_cast<const float2*>(state(in ? i0 + b : i0));
+      ml[b] = in ? __ldcg(p) : make_float2(-INFINITY, 0.f);
+#pragma unroll
+      for (int i = 0; i < V2; ++i) v[b][i] = in ? __ldcg(p + 1 + 4 * i + t) : make_float2(0.f, 0.f);
+    }
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const float w = (ml[b].x == -INFINITY) ? 0.f : exp2f(ml[b].x - Mc);
+      Lc = fmaf(ml[b].y, w, Lc);
+#pragma unroll
+      for (int i = 0; i < V2; ++i) {
+        o[i].x = fmaf(v[b][i].x, w, o[i].x);
+        o[i].y = fmaf(v[b][i].y, w, o[i].y);
+      }
+    }
+  }
+  if (!on) return;
+  const float inv = 1.f / Lc;
+#pragma unroll
+  for (int i = 0; i < V2; ++i)
+    *reinterpret_cast<uint32_t*>(ob + (size_t)g * D + 8 * i + 2 * t) = pack_bf16x2(o[i].x * inv, o[i].y * inv);
+}
+
 // kWin: the cache uses the window-grouping approximation (L.window > 0)
 template <int D, bool kWin>
 __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaArgs a) {
@@ -150,10 +218,15 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
     __threadfence_block();  // the prefix is read after its tag
   }
   const long long Utot = have_units ? U[NH] : 0;
-  const int NW = gridDim.x * kGWarps;
-  const int wid = blockIdx.x * kGWarps + warp;
-  const int u0 = have_units ? (int)range_start(wid, Utot, NW) : 0;
-  const int u1 = have_units ? (int)range_start(wid + 1, Utot, NW) : 0;
+  // The workers of the layer: every warp, or fewer when a head would then be
+  // cut into so many parts that merging them takes longer than streaming them
+  // (gqa_workers); those are spread over the blocks so that every SM takes part.
+  const int NWG = (int)gridDim.x * kGWarps;
+  const int NW = have_units ? gqa_workers(Utot, NH, NWG) : NWG;
+  const int wid = NW < NWG ? warp * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * kGWarps + warp;
+  const bool works = have_units && wid < NW;
+  const int u0 = works ? (int)range_start(wid, Utot, NW) : 0;
+  const int u1 = works ? (int)range_start(wid + 1, Utot, NW) : 0;
   const int n = u1 - u0;
   const uint32_t ring_s = smem_u32(ring);
 
@@ -538,55 +611,21 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
           __syncwarp();
           const int wf = worker_of_unit(hu0, Utot, NW);
           const int wl = worker_of_unit(hend - 1, Utot, NW);
-          const bool dense = Utot >= NW;
           int last = 0;
           if (lane == 0) {
-            int ncontrib = wl - wf + 1;
-            if (!dense) {
-              ncontrib = 0;
-              for (int cw = wf; cw <= wl; ++cw)
-                ncontrib += range_start(cw, Utot, NW) < range_start(cw + 1, Utot, NW);
-            }
+            // every worker in [wf, wl] holds part of the head
             int* cnt = L.counters + (size_t)layer * NH * G + vh;
             const int old = atomicAdd(cnt, 1);
-            last = (old == ncontrib - 1);
+            last = (old == wl - wf);
             if (last) *cnt = 0;
           }
           last = __shfl_sync(0xffffffffu, last, 0);
           if (last) {
-            __threadfence();
-            // lane: query g, a quarter of the dims
-            constexpr int DPQ = D / 4;
-            const int qq = g, d_lo = t * DPQ;
-            float Mc = -INFINITY;
-            for (int cw = wf; cw <= wl; ++cw) {
-              const long long cs0 = range_start(cw, Utot, NW);
-              if (cs0 == range_start(cw + 1, Utot, NW)) continue;
-              const int cs = 2 * cw + (hu0 <= cs0 ? 0 : 1);
-              if (qq < G) Mc = fmaxf(Mc, __ldcg(partials + ((size_t)cs * G + qq) * (D + 2)));
-            }
-            float Lc = 0.f, Oc[DPQ];
-#pragma unroll
-            for (int i = 0; i < DPQ; ++i) Oc[i] = 0.f;
-            for (int cw = wf; cw <= wl; ++cw) {
-              const long long cs0 = range_start(cw, Utot, NW);
-              if (cs0 == range_start(cw + 1, Utot, NW)) continue;
-              const int cs = 2 * cw + (hu0 <= cs0 ? 0 : 1);
-              if (qq < G) {
-                const float* cp = partials + ((size_t)cs * G + qq) * (D + 2);
-                const float mc = __ldcg(cp);
-                const float cwt = (mc == -INFINITY) ? 0.f : exp2f(mc - Mc);
-                Lc = fmaf(__ldcg(cp + 1), cwt, Lc);
-#pragma unroll
-                for (int i = 0; i < DPQ; ++i) Oc[i] = fmaf(__ldcg(cp + 2 + d_lo + i), cwt, Oc[i]);
-              }
-            }
-            if (qq < G) {
-              const float inv = 1.f / Lc;
-#pragma unroll
-              for (int i = 0; i < DPQ; ++i)
-                ob[(size_t)qq * D + d_lo + i] = __float2bfloat16_rn(Oc[i] * inv);
-            }
+            __threadfence();  // every contributor's states are visible to this lane
+            // worker wf + i wrote state 2 (wf + i) + 1 if the head starts
+            // inside its range (only possible for i = 0), else 2 (wf + i)
+            const int first_off = (hu0 > range_start(wf, Utot, NW)) ? 1 : 0;
+            combine_gqa<D>(partials, wf, first_off, wl - wf + 1, G, lane, ob);
           }
         }
         m = -INFINITY;
