@@ -16,12 +16,12 @@ cudaError_t decode_launch(const Layout& L, int layer0, int nlayers, int Gv, cons
 cudaError_t prefill_launch(const Layout& L, int layer, int first_seq, int num_seqs, const void* q,
                            long long q_tok, long long q_head, const void* k, const void* v,
                            const int* cu, int total_tokens, int max_seqlen, float* carry,
-                           cudaStream_t stream);
+                           float* weights, cudaStream_t stream);
 bool prefill_attn_supported(const Layout& L);
 cudaError_t prefill_attn_launch(const Layout& L, int layer, int first_seq, int num_seqs,
                                 const void* q, const void* k, const void* v, const int* cu,
-                                int total_tokens, int max_seqlen, const float* carry, void* out,
-                                cudaStream_t stream);
+                                int total_tokens, int max_seqlen, const float* carry,
+                                const float* weights, void* out, cudaStream_t stream);
 cudaError_t decode_static_partials(int device, float** ptr, size_t* floats);
 bool gqa_supported(const Layout& L);
 cudaError_t gqa_setup(const Layout& L, DecodePlan* plan);
@@ -47,7 +47,8 @@ struct dmc_cache {
   int last_decode_lo, last_decode_hi;  // layers [lo, hi) of the latest kernel if it was a decode, else empty
   char* meta;  // lengths, ctl, counters, pool top, error: cleared by create / reset
   size_t meta_bytes;
-  float* carry;  // segment sums at prompt chunk starts (prompt attention)
+  float* carry;    // segment sums at prompt chunk starts (prompt attention)
+  float* weights;  // decisions and omegas of the prompt's chunks (prompt attention)
 };
 
 namespace {
@@ -75,7 +76,7 @@ bool valid_config(const dmc_cache_config* c) {
 // Byte offsets of every region; returns the total size.
 struct Offsets {
   size_t pages, z, ptab, meta, lengths, ctl, counters, pool_top, error, meta_end, partials,
-      pending, pending_at, pending_z, opens, plan, carry, ring, ring_w, seglen, total;
+      pending, pending_at, pending_z, opens, plan, carry, weights, ring, ring_w, seglen, total;
   int MPH, plan_stride;
 };
 
@@ -114,6 +115,7 @@ Offsets offsets(const dmc_cache_config* c) {
   o.opens = at; at = align_up(at + (size_t)c->max_prefill_tokens * c->num_kv_heads);
   o.plan = at; at = align_up(at + (size_t)c->num_kv_heads * o.plan_stride * 4);
   o.carry = at; at = align_up(at + (size_t)o.plan_stride * c->num_kv_heads * (2 * c->head_dim + 1) * 4);
+  o.weights = at; at = align_up(at + (size_t)o.plan_stride * c->num_kv_heads * dmc::kPrefillChunk * 4);
   o.ring = at; at = align_up(at + (size_t)c->num_layers * NH * c->window * 2 * row);
   o.ring_w = at; at = align_up(at + (size_t)c->num_layers * NH * c->window * 4);
   o.total = at;
@@ -213,6 +215,7 @@ dmc_status dmc_cache_create(const dmc_cache_config* cfg, void* arena_dev, size_t
   L.plan = reinterpret_cast<int*>(base + o.plan);
   L.plan_stride = o.plan_stride;
   c->carry = reinterpret_cast<float*>(base + o.carry);
+  c->weights = reinterpret_cast<float*>(base + o.weights);
   L.window = cfg->window;
   L.ring = cfg->window > 0 ? base + o.ring : nullptr;
   L.ring_w = cfg->window > 0 ? reinterpret_cast<float*>(base + o.ring_w) : nullptr;
@@ -279,7 +282,7 @@ dmc_status dmc_prefill_compress(dmc_cache_t c, int32_t layer, int32_t first_seq,
   no_pdl_next(c);
   return cuda_status(dmc::prefill_launch(L, layer, first_seq, num_seqs, q_dev, q_token_stride,
                                          q_head_stride, k_dev, v_dev, cu_seqlens_dev, total_tokens,
-                                         max_seqlen, nullptr, stream));
+                                         max_seqlen, nullptr, nullptr, stream));
 }
 
 dmc_status dmc_prefill_attention(dmc_cache_t c, int32_t layer, int32_t first_seq,
@@ -303,11 +306,11 @@ dmc_status dmc_prefill_attention(dmc_cache_t c, int32_t layer, int32_t first_seq
   const long long q_tok = (long long)L.Hq * L.D, q_head = L.D;
   cudaError_t e = dmc::prefill_launch(L, layer, first_seq, num_seqs, q_dev, q_tok, q_head, k_dev,
                                       v_dev, cu_seqlens_dev, total_tokens, max_seqlen, c->carry,
-                                      stream);
+                                      c->weights, stream);
   if (e != cudaSuccess) return DMC_ERR_CUDA;
   return cuda_status(dmc::prefill_attn_launch(L, layer, first_seq, num_seqs, q_dev, k_dev, v_dev,
                                               cu_seqlens_dev, total_tokens, max_seqlen, c->carry,
-                                              out_dev, stream));
+                                              c->weights, out_dev, stream));
 }
 
 dmc_status dmc_decode_step(dmc_cache_t c, int32_t layer, const void* q_dev, const void* k_dev,

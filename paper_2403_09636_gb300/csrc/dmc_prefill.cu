@@ -40,7 +40,8 @@ struct PrefillArgs {
   const char* v;
   const int* cu;
   int total_tokens, max_seqlen;
-  float* carry;  // [chunk id][Hkv][2D + 1] (sum w k, sum w v, sum w), or null
+  float* carry;    // [chunk id][Hkv][2D + 1] (sum w k, sum w v, sum w), or null
+  float* weights;  // with carry: [chunk id][Hkv][128], omega, negative where the token opens a slot
 };
 
 __device__ __forceinline__ bool seq_bounds(const PrefillArgs& a, int s, int& t0, int& t1) {
@@ -358,10 +359,20 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   const unsigned char* op = L.opens + h;
   const size_t ostride = (size_t)L.Hkv;
   const T* qq = reinterpret_cast<const T*>(a.q);
-  auto omega = [&](int t) {  // omega = sigmoid(q[0]) (group mean for GQA)
-    float y = 0.f;
-    for (int gq = 0; gq < L.G; ++gq)
-      y += Elt<T>::to_f(qq[(size_t)t * a.q_tok + (size_t)(h * L.G + gq) * a.q_head]);
+  // omega = sigmoid(q[0]) (group mean for GQA); the group's loads, up to eight
+  // at a time, are in flight together
+  auto omega = [&](int t) {
+    const T* q0 = qq + (size_t)t * a.q_tok + (size_t)(h * L.G) * a.q_head;
+    float y = Elt<T>::to_f(q0[0]);
+    for (int g0 = 1; g0 < L.G; g0 += 7) {
+      T x[7];
+#pragma unroll
+      for (int u = 0; u < 7; ++u)
+        if (g0 + u < L.G) x[u] = q0[(size_t)(g0 + u) * a.q_head];
+#pragma unroll
+      for (int u = 0; u < 7; ++u)
+        if (g0 + u < L.G) y += Elt<T>::to_f(x[u]);
+    }
     return sigmoidf_(y / (float)L.G);
   };
   // pages of the slots the block may write, [base - 1, base + 128): at most
@@ -375,7 +386,10 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     const int t = a0 + tid, tn = a1 + tid;
     const bool f = t < a1 && op[(size_t)t * ostride];
     const bool fn = tn < t1 && op[(size_t)tn * ostride];
-    s_w[tid] = t < a1 ? omega(t) : 0.f;
+    const float w = t < a1 ? omega(t) : 0.f;
+    s_w[tid] = w;
+    if (a.weights != nullptr)
+      a.weights[((size_t)chunk_id(t0, c, s) * L.Hkv + h) * kPrefillChunk + tid] = f ? -w : w;
     const unsigned bal = __ballot_sync(0xffffffffu, f), nbal = __ballot_sync(0xffffffffu, fn);
     if (lane == 0) { s_bal[warp] = bal; s_nbal[warp] = nbal; }
   }
@@ -704,7 +718,7 @@ static cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t stream) {
 cudaError_t prefill_launch(const Layout& L, int layer, int first_seq, int num_seqs, const void* q,
                            long long q_tok, long long q_head, const void* k, const void* v,
                            const int* cu, int total_tokens, int max_seqlen, float* carry,
-                           cudaStream_t stream) {
+                           float* weights, cudaStream_t stream) {
   PrefillArgs a;
   a.lay = L;
   a.layer = layer;
@@ -719,6 +733,7 @@ cudaError_t prefill_launch(const Layout& L, int layer, int first_seq, int num_se
   a.total_tokens = total_tokens;
   a.max_seqlen = max_seqlen;
   a.carry = carry;
+  a.weights = weights;
   if (L.esize == 4 && L.D == 64) return launch_prefill<float, 64>(a, stream);
   if (L.esize == 4 && L.D == 128) return launch_prefill<float, 128>(a, stream);
   if (L.esize == 2 && L.D == 64) return launch_prefill<__nv_bfloat16, 64>(a, stream);
