@@ -15,9 +15,8 @@
 //        that continue the head's existing last slot); a segment that runs past
 //        the chunk end is followed to its end. Lanes split a row into 16-byte
 //        pieces and accumulate sum(omega k), sum(omega v), sum(omega) in fp32;
-//        the slot is the quotient, rounded once to the cache dtype. Exact
-//        compression walks the chunk's tokens in row groups (see the kernel);
-//        window grouping gives each segment to one warp. When asked for
+//        the slot is the quotient, rounded once to the cache dtype. The chunk's
+//        tokens are walked in row groups (see the kernel). When asked for
 //        (prompt attention), the block also records, at every chunk start a
 //        segment runs across, the segment's sums up to that point (the
 //        "carry"), so that each chunk can rebuild the running state of its
@@ -152,98 +151,6 @@ __device__ __forceinline__ float* carry_at(const PrefillArgs& a, int t0, int cs,
   return a.carry + ((size_t)chunk_id(t0, (cs - t0) / kPrefillChunk, s) * a.lay.Hkv + h) * (2 * D + 1);
 }
 
-// Window grouping: one warp sums segment [tb, te) into `slot`, counting only
-// its last W tokens; the head's open segment keeps its last W - 1 tokens in
-// the ring (token p of the segment at entry p % W) and its length in seglen,
-// and a prompt that continues it (merge_old) takes the continued segment's
-// tokens still inside the window from there.
-template <typename T, int D>
-__device__ __noinline__ void scan_window_segment(const PrefillArgs& a, int h, int bh, int tb,
-                                                 int te, int slot, bool merge_old) {
-  using CK = Chunk<T>;
-  constexpr int ROW = D * (int)sizeof(T);
-  constexpr int LPR = ROW / 16;  // lanes per row
-  constexpr int RPI = 32 / LPR;  // rows per warp iteration
-  constexpr int EPC = CK::N;
-  const Layout& L = a.lay;
-  const int lane = threadIdx.x & 31, sub = lane / LPR, lr = lane % LPR;
-  const T* qq = reinterpret_cast<const T*>(a.q);
-  float ak[EPC], av[EPC], zs = 0.f;
-#pragma unroll
-  for (int e = 0; e < EPC; ++e) { ak[e] = 0.f; av[e] = 0.f; }
-  const int page = L.page_table[((size_t)a.layer * L.NH + bh) * L.MPH + slot / kPage];
-  char* kdst = L.pages + (size_t)page * L.page_bytes + (size_t)(slot % kPage) * ROW + lr * 16;
-  char* vdst = kdst + (size_t)kPage * ROW;
-  float* zp = L.z + (size_t)page * kPage + slot % kPage;
-  const int W = L.window;
-  const int parity = *reinterpret_cast<const volatile int*>(&L.ctl[a.layer * 4]);
-  const char* ring = L.ring + ((size_t)a.layer * L.NH + bh) * W * 2 * ROW;
-  const float* ring_w = L.ring_w + ((size_t)a.layer * L.NH + bh) * W;
-  if (merge_old && sub == 0) {
-    // the continued segment's tokens still inside the window, from the ring
-    const int n_old = L.seglen[((size_t)a.layer * 2 + parity) * L.NH + bh];
-    const int m = min(n_old, max(0, W - (te - tb)));
-    for (int e = 0; e < m; ++e) {
-      const int pos = (n_old - 1 - e) % W;
-      float ko[EPC], vo[EPC];
-      CK::unpack(*reinterpret_cast<const uint4*>(ring + (size_t)pos * 2 * ROW + lr * 16), ko);
-      CK::unpack(*reinterpret_cast<const uint4*>(ring + (size_t)pos * 2 * ROW + ROW + lr * 16), vo);
-      const float w = ring_w[pos];
-#pragma unroll
-      for (int e2 = 0; e2 < EPC; ++e2) {
-        ak[e2] = fmaf(w, ko[e2], ak[e2]);
-        av[e2] = fmaf(w, vo[e2], av[e2]);
-      }
-      if (lr == 0) zs += w;
-    }
-  }
-  const size_t hrow = (size_t)L.Hkv * ROW;
-  const char* kb = a.k + (size_t)h * ROW + lr * 16;
-  const char* vb = a.v + (size_t)h * ROW + lr * 16;
-#pragma unroll 2
-  for (int t = max(tb, te - W) + sub; t < te; t += RPI) {  // the segment's last W tokens
-    const uint4 kr = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)t * hrow));
-    const uint4 vr = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)t * hrow));
-    float y = 0.f;
-    for (int g = 0; g < L.G; ++g)
-      y += Elt<T>::to_f(qq[(size_t)t * a.q_tok + (size_t)(h * L.G + g) * a.q_head]);
-    const float w = sigmoidf_(y / (float)L.G);  // omega = sigmoid(q[0]) (group mean for GQA)
-    float kf[EPC], vf[EPC];
-    CK::unpack(kr, kf);
-    CK::unpack(vr, vf);
-    if (lr == 0) kf[0] = 0.f;  // k[0] <- 0 (Algorithm 1)
-#pragma unroll
-    for (int e = 0; e < EPC; ++e) {
-      ak[e] = fmaf(w, kf[e], ak[e]);
-      av[e] = fmaf(w, vf[e], av[e]);
-    }
-    zs += w;
-  }
-#pragma unroll
-  for (int off = LPR; off < 32; off <<= 1) {
-#pragma unroll
-    for (int e = 0; e < EPC; ++e) {
-      ak[e] += __shfl_xor_sync(0xffffffffu, ak[e], off);
-      av[e] += __shfl_xor_sync(0xffffffffu, av[e], off);
-    }
-    zs += __shfl_xor_sync(0xffffffffu, zs, off);
-  }
-  // the lr == 0 lane holds z; every lane needs it for the quotient
-  zs = __shfl_sync(0xffffffffu, zs, lane - lr);
-  if (sub != 0) return;
-  const float iz = 1.f / zs;
-  float kn[EPC], vn[EPC];
-#pragma unroll
-  for (int e = 0; e < EPC; ++e) {
-    kn[e] = ak[e] * iz;
-    vn[e] = av[e] * iz;
-  }
-  if (lr == 0) kn[0] = 0.f;
-  *reinterpret_cast<uint4*>(kdst) = CK::pack(kn);
-  *reinterpret_cast<uint4*>(vdst) = CK::pack(vn);
-  if (lr == 0) *zp = zs;
-}
-
 // Window grouping: the head's open segment [tb, te = end of the prompt), which
 // had n_old tokens before this prompt, leaves its last W - 1 tokens (k with
 // k[0] cleared, v, omega) in the ring and its length in seglen. One warp.
@@ -297,8 +204,17 @@ constexpr int kRing = 8;        // rows in a lane's ring
 constexpr int kRingBatch = 4;   // rows per async-copy group
 constexpr size_t kScanRingBytes = (size_t)kRing * 2 * kScanThreads * 16;
 
-template <typename T, int D>
-__global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const PrefillArgs a) {
+//
+// Window grouping (kWin): a slot counts only its segment's last W tokens. A
+// segment of at most W tokens is summed as above; of a longer one the last W
+// rows are read again when it ends (they are in L2: a longer segment costs at
+// most one more read of its rows), and one that continues the head's last slot
+// takes the old tokens still inside the window from the head's ring (token p of
+// the segment at entry p % W). With the spill-free 128 registers (4 blocks per SM)
+// plan + scan of a 7B layer (32 x 2048 tokens at 4x, W = 12) takes 380 us; one warp
+// per segment, rows straight into registers, took 883.
+template <typename T, int D, bool kWin>
+__global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_kernel(const PrefillArgs a) {
   using CK = Chunk<T>;
   constexpr int ROW = D * (int)sizeof(T);
   constexpr int LPR = ROW / 16;               // lanes per row
@@ -456,6 +372,28 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     *reinterpret_cast<uint4*>(kdst + (size_t)kPage * ROW) = CK::pack(vn);
     if (lr == 0) L.z[(size_t)s_page[slot / kPage - pfirst] * kPage + slot % kPage] = zs;
   };
+  // window grouping: the sums of segment [tb, te), if it is longer than the window
+  auto window_sums = [&](int tb, int te) {
+    const int W = L.window;
+    if (te - tb <= W) return;
+    reset();
+#pragma unroll 1
+    for (int t = te - W; t < te; t += 4) {
+      uint4 kr[4], vr[4];
+      float w[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (t + u < te) {
+          kr[u] = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)(t + u) * hrow));
+          vr[u] = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)(t + u) * hrow));
+          w[u] = t + u < a1 && t + u >= a0 ? s_w[t + u - a0] : omega(t + u);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (t + u < te) add_row(kr[u], vr[u], w[u]);
+    }
+  };
   auto group_bits = [&](int gg) {  // the opening tokens of group gg's range
     const unsigned b = s_bal[(gg * TPG) >> 5] >> ((gg * TPG) & 31);
     return TPG == 32 ? b : (b & ((1u << TPG) - 1u));
@@ -473,6 +411,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   }
   float hk[EPC], hv[EPC], hz = 0.f;  // the sums before the group's first opening
   bool open = false;                 // summing a segment that opened in this group
+  int opened = 0;                    // ... at this token (window grouping)
   reset();
   for (int b = 0; b < NB; ++b) {
     cp_async_wait<1>();  // copy group b has landed
@@ -482,6 +421,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
       if (t >= wb && t < g1) {
         if ((gbits >> (t - g0)) & 1u) {  // t opens a slot: the segment before it ends
           if (open) {
+            if constexpr (kWin) window_sums(opened, t);
             write_slot(slot);
           } else {
 #pragma unroll
@@ -490,6 +430,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
           }
           reset();
           open = true;
+          if constexpr (kWin) opened = t;
           ++slot;
         }
         const uint32_t sk = rk((b % 2) * kRingBatch + u);
@@ -564,88 +505,63 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
       }
     }
   };
+  // where the segment that is open at the end of group gg ends
+  auto segment_end = [&](int gg) {
+    for (++gg; gg < NG; ++gg)
+      if (const unsigned bits = group_bits(gg)) return a0 + gg * TPG + __ffs(bits) - 1;
+    return next;
+  };
   // job 0: the group's open segment (its sums are in the registers); job 1
   // (group 0 of chunk 0 only): the segment that continues the head's last slot
   const int jobs_end = (pre && g == 0) ? 2 : 1;
   for (int job = open ? 0 : 1; job < jobs_end; ++job) {
     int from = g;
     if (job == 1) {
-      // the old slot's K z_old, V z_old and z_old start the sums
       slot = base - 1;
       from = -1;
-      const char* kold = slot_ptr(slot);
-      float ko[EPC], vo[EPC];
-      CK::unpack(*reinterpret_cast<const uint4*>(kold), ko);
-      CK::unpack(*reinterpret_cast<const uint4*>(kold + (size_t)kPage * ROW), vo);
-      const float zo = L.z[(size_t)s_page[slot / kPage - pfirst] * kPage + slot % kPage];
-#pragma unroll
-      for (int e = 0; e < EPC; ++e) {
-        ak[e] = ko[e] * zo;
-        av[e] = vo[e] * zo;
+    }
+    if constexpr (kWin) {
+      const int W = L.window, tb = job == 1 ? t0 : opened, te = segment_end(from);
+      if (te - tb > W) {
+        window_sums(tb, te);
+        write_slot(slot);
+        continue;
       }
-      zs = zo;
-      if (carry) put_carry(t0);  // the state the prompt's first token continues
+    }
+    if (job == 1) {
+      if constexpr (kWin) {
+        // the continued segment's tokens still inside the window
+        reset();
+        const int W = L.window, te = segment_end(from);
+        const int parity = *reinterpret_cast<const volatile int*>(&L.ctl[a.layer * 4]);
+        const int n_old = L.seglen[((size_t)a.layer * 2 + parity) * L.NH + bh];
+        const int m = min(n_old, W - (te - t0));
+        const char* old = L.ring + ((size_t)a.layer * L.NH + bh) * W * 2 * ROW + lr * 16;
+        const float* old_w = L.ring_w + ((size_t)a.layer * L.NH + bh) * W;
+#pragma unroll 2
+        for (int e = 0; e < m; ++e) {
+          const int pos = (n_old - 1 - e) % W;
+          add_row(*reinterpret_cast<const uint4*>(old + (size_t)pos * 2 * ROW),
+                  *reinterpret_cast<const uint4*>(old + (size_t)pos * 2 * ROW + ROW), old_w[pos]);
+        }
+      } else {
+        // the old slot's K z_old, V z_old and z_old start the sums
+        const char* kold = slot_ptr(slot);
+        float ko[EPC], vo[EPC];
+        CK::unpack(*reinterpret_cast<const uint4*>(kold), ko);
+        CK::unpack(*reinterpret_cast<const uint4*>(kold + (size_t)kPage * ROW), vo);
+        const float zo = L.z[(size_t)s_page[slot / kPage - pfirst] * kPage + slot % kPage];
+#pragma unroll
+        for (int e = 0; e < EPC; ++e) {
+          ak[e] = ko[e] * zo;
+          av[e] = vo[e] * zo;
+        }
+        zs = zo;
+        if (carry) put_carry(t0);  // the state the prompt's first token continues
+      }
     }
     finish(from);
     write_slot(slot);
-  }
-}
-
-// Window grouping: one warp per segment (the slot counts only the segment's
-// last W tokens, and a continued segment's old tokens come from the ring).
-template <typename T, int D>
-__global__ void __launch_bounds__(kScanThreads) dmc_prefill_scan_window_kernel(const PrefillArgs a) {
-  __shared__ int starts[kPrefillChunk];
-  __shared__ int s_wcnt[kScanThreads / 32];
-  __shared__ int s_next;
-  const Layout& L = a.lay;
-  const int c = blockIdx.x, h = blockIdx.y, s = blockIdx.z;
-  const int bh = (a.first_seq + s) * L.Hkv + h;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int t0, t1;
-  if (!seq_bounds(a, s, t0, t1)) return;
-  const int a0 = t0 + c * kPrefillChunk;
-  if (a0 >= t1) return;
-  const int a1 = min(a0 + kPrefillChunk, t1);
-  const int base = L.plan[(size_t)h * L.plan_stride + chunk_id(t0, c, s)];
-  if (base < 0) return;
-  const unsigned char* op = L.opens + h;
-  const size_t ostride = (size_t)L.Hkv;
-
-  // positions of the tokens of [a0, a1) that open a slot, in order
-  static_assert(kScanThreads == kPrefillChunk, "one thread per chunk token");
-  const int t = a0 + tid;
-  const bool f = (t < a1) && op[(size_t)t * ostride];
-  const unsigned bal = __ballot_sync(0xffffffffu, f);
-  if (lane == 0) s_wcnt[warp] = __popc(bal);
-  if (tid == 0) s_next = t1;
-  __syncthreads();
-  int before = __popc(bal & ((1u << lane) - 1u));
-  for (int w = 0; w < warp; ++w) before += s_wcnt[w];
-  int nstart = 0;
-  for (int w = 0; w < kScanThreads / 32; ++w) nstart += s_wcnt[w];
-  if (f) starts[before] = t;
-  // the first opening token at or after a1 ends the chunk's last segment
-  for (int b0 = a1; b0 < t1; b0 += kScanThreads) {
-    const int tt = b0 + tid;
-    const bool g = tt < t1 && op[(size_t)tt * ostride];
-    if (g) atomicMin(&s_next, tt);
-    if (__syncthreads_or(g)) break;
-  }
-  __syncthreads();
-  const int next = s_next;
-  const bool pre = (c == 0) && !op[(size_t)t0 * ostride];  // continues the existing last slot
-  const int items = nstart + (pre ? 1 : 0);
-  for (int it = warp; it < items; it += kScanThreads / 32) {
-    if (pre && it == 0) {
-      const int te = nstart > 0 ? starts[0] : next;
-      scan_window_segment<T, D>(a, h, bh, t0, te, base - 1, true);
-    } else {
-      const int j = it - (pre ? 1 : 0);
-      const int tb = starts[j];
-      const int te = (j + 1 < nstart) ? starts[j + 1] : next;
-      scan_window_segment<T, D>(a, h, bh, tb, te, base + j, false);
-    }
   }
 }
 
@@ -691,21 +607,18 @@ static cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t stream) {
   if (e != cudaSuccess) return e;
   if (max_chunks > 0) {
     const dim3 grid(max_chunks, a.lay.Hkv, a.num_seqs);
-    if (a.lay.window > 0) {
-      dmc_prefill_scan_window_kernel<T, D><<<grid, kScanThreads, 0, stream>>>(a);
-    } else {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = grid;
-      cfg.blockDim = dim3(kScanThreads);
-      cfg.stream = stream;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[0].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      e = cudaLaunchKernelEx(&cfg, dmc_prefill_scan_kernel<T, D>, a);
-      if (e != cudaSuccess) return e;
-    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kScanThreads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = a.lay.window > 0 ? cudaLaunchKernelEx(&cfg, dmc_prefill_scan_kernel<T, D, true>, a)
+                         : cudaLaunchKernelEx(&cfg, dmc_prefill_scan_kernel<T, D, false>, a);
+    if (e != cudaSuccess) return e;
     e = cudaGetLastError();
   }
   if (e == cudaSuccess && a.lay.window > 0) {
