@@ -201,6 +201,11 @@ __device__ __forceinline__ void fill_ring(const PrefillArgs& a, int h, int bh, i
 // at each chunk start it runs across), and chunk 0 also finishes the segment
 // that continues the head's existing last slot.
 constexpr int kRing = 8;        // rows in a lane's ring
+// Rows of a segment past its chunk that its group still adds alone, two at a time
+// (7B at 4x: three on average). More are summed by all groups: at CR 32 plan + scan
+// of 32 x 2048 tokens takes 289 us, with one group for any tail 477; at 4x the
+// exchange costs more than it saves (297 us if every tail is shared, 281 so).
+constexpr int kLongTail = 8;
 constexpr int kRingBatch = 4;   // rows per async-copy group
 constexpr size_t kScanRingBytes = (size_t)kRing * 2 * kScanThreads * 16;
 
@@ -227,7 +232,7 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
   static_assert(kScanThreads == kPrefillChunk, "one thread per chunk token");
   static_assert(TPG <= 32 && 32 % TPG == 0, "a group's tokens sit in one ballot word");
   static_assert(kRing == 2 * kRingBatch, "two copy groups in flight");
-  static_assert((size_t)NG * HS * sizeof(float) <= kScanRingBytes, "heads fit the ring");
+  static_assert((size_t)2 * NG * HS * sizeof(float) <= kScanRingBytes, "heads and tails fit the ring");
   __shared__ __align__(16) unsigned char ring[kScanRingBytes];  // [kRing][K, V][thread] 16 B
   __shared__ float s_w[kPrefillChunk];
   __shared__ unsigned s_bal[kPrefillChunk / 32], s_nbal[kPrefillChunk / 32];
@@ -342,18 +347,25 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
     for (int e = 0; e < EPC; ++e) { ak[e] = 0.f; av[e] = 0.f; }
     zs = 0.f;
   };
-  auto add_row = [&](const uint4& kr, const uint4& vr, float w) {
+  auto add_to = [&](float* xk, float* xv, float& xz, const uint4& kr, const uint4& vr, float w) {
     float kf[EPC], vf[EPC];
     CK::unpack(kr, kf);
     CK::unpack(vr, vf);
     if (lr == 0) kf[0] = 0.f;  // k[0] <- 0 (Algorithm 1)
+    const float2 ww = make_float2(w, w);
 #pragma unroll
-    for (int e = 0; e < EPC; ++e) {
-      ak[e] = fmaf(w, kf[e], ak[e]);
-      av[e] = fmaf(w, vf[e], av[e]);
+    for (int e = 0; e < EPC; e += 2) {
+      const float2 sk = fma2(ww, make_float2(kf[e], kf[e + 1]), make_float2(xk[e], xk[e + 1]));
+      const float2 sv = fma2(ww, make_float2(vf[e], vf[e + 1]), make_float2(xv[e], xv[e + 1]));
+      xk[e] = sk.x; xk[e + 1] = sk.y;
+      xv[e] = sv.x; xv[e + 1] = sv.y;
     }
-    zs += w;
+    xz += w;
   };
+  auto add_row = [&](const uint4& kr, const uint4& vr, float w) { add_to(ak, av, zs, kr, vr, w); };
+  // The chunk's last segment runs on to `next`. Few rows there are its group's
+  // work, two at a time; more are summed by all groups, 128 tokens at a time.
+  const bool long_tail = next - a1 > kLongTail && (!kWin || next - a1 < L.window);
   auto slot_ptr = [&](int slot) {
     const int page = s_page[slot / kPage - pfirst];
     return L.pages + (size_t)page * L.page_bytes + (size_t)(slot % kPage) * ROW + lr * 16;
@@ -454,12 +466,53 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
   cp_async_wait<0>();
   __syncthreads();
   float* heads = reinterpret_cast<float*>(ring);
+  float* tails = heads + NG * HS;
+  auto put = [&](float* to) {
 #pragma unroll
-  for (int e = 0; e < EPC; ++e) {
-    heads[g * HS + lr * EPC + e] = hk[e];
-    heads[g * HS + D + lr * EPC + e] = hv[e];
+    for (int e = 0; e < EPC; ++e) {
+      to[g * HS + lr * EPC + e] = hk[e];
+      to[g * HS + D + lr * EPC + e] = hv[e];
+    }
+    if (lr == 0) to[g * HS + 2 * D] = hz;
+  };
+  auto add = [&](const float* from) {
+#pragma unroll
+    for (int e = 0; e < EPC; ++e) {
+      ak[e] += from[lr * EPC + e];
+      av[e] += from[D + lr * EPC + e];
+    }
+    zs += from[2 * D];
+  };
+  // adds the rows t0, t0 + step, ... below te
+  auto add_rows = [&](float* xk, float* xv, float& xz, int tb, int step, int te) {
+#pragma unroll 1
+    for (int t = tb; t < te; t += 2 * step) {
+      uint4 kr[2], vr[2];
+      float w[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        if (t + u * step < te) {
+          kr[u] = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)(t + u * step) * hrow));
+          vr[u] = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)(t + u * step) * hrow));
+          w[u] = omega(t + u * step);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (t + u * step < te) add_to(xk, xv, xz, kr[u], vr[u], w[u]);
+    }
+  };
+  auto tail_sums = [&](int pb) {  // this group's rows among [pb, min(next, pb + 128))
+#pragma unroll
+    for (int e = 0; e < EPC; ++e) { hk[e] = 0.f; hv[e] = 0.f; }
+    hz = 0.f;
+    add_rows(hk, hv, hz, pb + g, NG, min(next, pb + kPrefillChunk));
+  };
+  put(heads);
+  if (long_tail) {
+    tail_sums(a1);
+    put(tails);
   }
-  if (lr == 0) heads[g * HS + 2 * D] = hz;
   __syncthreads();
 
   const bool carry = a.carry != nullptr;
@@ -473,37 +526,21 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
     if (lr == 0) cp[2 * D] = zs;
   };
   // adds the heads of the groups after gg up to the first with an opening; if
-  // none has one, the segment is the chunk's last and runs on to `next`
-  auto finish = [&](int gg) {
+  // none has one, the segment is the chunk's last and runs on to `next`: true,
+  // after its rows in the 128 tokens from a1 have been added
+  auto finish = [&](int gg) -> bool {
     for (++gg; gg < NG; ++gg) {
-      const float* hp = heads + gg * HS;
-#pragma unroll
-      for (int e = 0; e < EPC; ++e) {
-        ak[e] += hp[lr * EPC + e];
-        av[e] += hp[D + lr * EPC + e];
-      }
-      zs += hp[2 * D];
-      if (group_bits(gg)) return;
+      add(heads + gg * HS);
+      if (group_bits(gg)) return false;
     }
-    for (int pb = a1; pb < next; pb += kPrefillChunk) {
-      if (carry) put_carry(pb);  // the segment runs across the chunk starting at pb
-      const int pe = min(next, pb + kPrefillChunk);
-      for (int tb = pb; tb < pe; tb += 2) {
-        uint4 kr[2], vr[2];
-        float w[2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          if (tb + u < pe) {
-            kr[u] = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)(tb + u) * hrow));
-            vr[u] = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)(tb + u) * hrow));
-            w[u] = omega(tb + u);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-          if (tb + u < pe) add_row(kr[u], vr[u], w[u]);
-      }
+    if (next > a1 && carry) put_carry(a1);
+    if (long_tail) {
+#pragma unroll 1
+      for (int i = 0; i < NG; ++i) add(tails + i * HS);
+    } else {
+      add_rows(ak, av, zs, a1, 1, next);
     }
+    return true;
   };
   // where the segment that is open at the end of group gg ends
   auto segment_end = [&](int gg) {
@@ -511,28 +548,27 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
       if (const unsigned bits = group_bits(gg)) return a0 + gg * TPG + __ffs(bits) - 1;
     return next;
   };
-  // job 0: the group's open segment (its sums are in the registers); job 1
-  // (group 0 of chunk 0 only): the segment that continues the head's last slot
-  const int jobs_end = (pre && g == 0) ? 2 : 1;
-  for (int job = open ? 0 : 1; job < jobs_end; ++job) {
-    int from = g;
-    if (job == 1) {
-      slot = base - 1;
-      from = -1;
+  // The segment that continues the head's last slot is group 0's work (of chunk
+  // 0); with an opening in the chunk group 0 may have one of its own besides,
+  // whose sums it puts aside.
+  const bool both = pre && g == 0 && nstart > 0 && open;
+  bool mine = open, past = false;
+  if (pre && g == 0) {
+    const int own_slot = slot;
+    if (both) {
+#pragma unroll
+      for (int e = 0; e < EPC; ++e) { hk[e] = ak[e]; hv[e] = av[e]; }
+      hz = zs;
     }
-    if constexpr (kWin) {
-      const int W = L.window, tb = job == 1 ? t0 : opened, te = segment_end(from);
-      if (te - tb > W) {
-        window_sums(tb, te);
-        write_slot(slot);
-        continue;
-      }
-    }
-    if (job == 1) {
+    slot = base - 1;
+    const int te = segment_end(-1);
+    if (kWin && te - t0 > L.window) {
+      window_sums(t0, te);
+    } else {
       if constexpr (kWin) {
         // the continued segment's tokens still inside the window
         reset();
-        const int W = L.window, te = segment_end(from);
+        const int W = L.window;
         const int parity = *reinterpret_cast<const volatile int*>(&L.ctl[a.layer * 4]);
         const int n_old = L.seglen[((size_t)a.layer * 2 + parity) * L.NH + bh];
         const int m = min(n_old, W - (te - t0));
@@ -559,10 +595,42 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
         zs = zo;
         if (carry) put_carry(t0);  // the state the prompt's first token continues
       }
+      past = finish(-1);
     }
-    finish(from);
-    write_slot(slot);
+    if (nstart > 0) {
+      write_slot(slot);
+      past = false;
+      slot = own_slot;
+      if (both) {
+#pragma unroll
+        for (int e = 0; e < EPC; ++e) { ak[e] = hk[e]; av[e] = hv[e]; }
+        zs = hz;
+      }
+    } else {
+      mine = true;  // the chunk's only segment: below
+    }
   }
+  if (open) {
+    const int te = kWin ? segment_end(g) : 0;
+    if (kWin && te - opened > L.window) {
+      window_sums(opened, te);
+    } else {
+      past = finish(g);
+    }
+  }
+  if constexpr (!kWin) {
+    // a segment that runs on beyond the 128 tokens from a1
+    for (int pb = a1 + kPrefillChunk; pb < next; pb += kPrefillChunk) {
+      if (past && carry) put_carry(pb);
+      tail_sums(pb);
+      __syncthreads();  // the tails before have been read
+      put(tails);
+      __syncthreads();
+      if (past)
+        for (int i = 0; i < NG; ++i) add(tails + i * HS);
+    }
+  }
+  if (mine) write_slot(slot);
 }
 
 // Window grouping: after the scan (which read the old window of continued

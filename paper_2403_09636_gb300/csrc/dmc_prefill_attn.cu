@@ -189,24 +189,6 @@ __device__ __forceinline__ float pa_ex2(float x) {
   return y;
 }
 
-// two fp32 operations in one instruction
-__device__ __forceinline__ float2 pa_fma2(float2 a, float2 b, float2 c) {
-  float2 d;
-  asm("{\n\t.reg .b64 x, y, z, w;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
-      "fma.rn.f32x2 w, x, y, z;\n\tmov.b64 {%0, %1}, w;\n\t}"
-      : "=f"(d.x), "=f"(d.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-  return d;
-}
-__device__ __forceinline__ float2 pa_add2(float2 a, float2 b) {
-  float2 d;
-  asm("{\n\t.reg .b64 x, y, w;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\t"
-      "add.rn.f32x2 w, x, y;\n\tmov.b64 {%0, %1}, w;\n\t}"
-      : "=f"(d.x), "=f"(d.y)
-      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-  return d;
-}
-
 __device__ __forceinline__ void pa_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                    bar)
@@ -867,9 +849,9 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
           uint32_t pk[32];
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
-            const float2 x = pa_fma2(make_float2(s[c0 + 2 * i], s[c0 + 2 * i + 1]), scale2, shift2);
+            const float2 x = fma2(make_float2(s[c0 + 2 * i], s[c0 + 2 * i + 1]), scale2, shift2);
             const float2 p = make_float2(pa_ex2(x.x), pa_ex2(x.y));
-            sum[i & 1] = pa_add2(sum[i & 1], p);
+            sum[i & 1] = add2(sum[i & 1], p);
             pk[i] = Chunk<__nv_bfloat16>::pack2(p.x, p.y);
           }
           // P over the row's own S columns: slots c0 + 2 i, + 1 in column c0 / 2 + i
