@@ -228,6 +228,14 @@ dmc_status dmc_cache_export_heads(dmc_cache_t cache, int32_t layer, int32_t n,
                                   void* v_out_dev, float* z_out_dev, int32_t* len_out_dev,
                                   cudaStream_t stream);
 
+/* dmc_cache_export_heads into buffers that need not be cleared first: the rows
+ * from a head's count to cap (all rows of a head id that does not exist, whose
+ * len_out_dev is -1) are set to zero in the same pass. */
+dmc_status dmc_cache_export_heads_padded(dmc_cache_t cache, int32_t layer, int32_t n,
+                                         const int32_t* head_ids_dev, int32_t cap, void* k_out_dev,
+                                         void* v_out_dev, float* z_out_dev, int32_t* len_out_dev,
+                                         cudaStream_t stream);
+
 /* Synchronizes `stream`, then reads the sticky fault bits (into *bits if not
  * NULL) and the number of pool pages handed out so far (into *pages_used if
  * not NULL). Returns DMC_OK, DMC_ERR_PAGES_EXHAUSTED or DMC_ERR_DEVICE_FAULT. */

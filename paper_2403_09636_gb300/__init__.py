@@ -32,7 +32,7 @@ PAGE_SIZE = 32
 EXPORTED = ("dmc_cache_required_bytes", "dmc_cache_create", "dmc_cache_destroy",
             "dmc_cache_reset", "dmc_prefill_compress", "dmc_prefill_attention", "dmc_decode_step",
             "dmc_decode_step_layers", "dmc_decode_step_static_scratch", "dmc_cache_lengths",
-            "dmc_cache_export_heads", "dmc_cache_status", "dmc_status_string")
+            "dmc_cache_export_heads", "dmc_cache_export_heads_padded", "dmc_cache_status", "dmc_status_string")
 
 
 class dmc_cache_config(C.Structure):
@@ -76,6 +76,7 @@ def lib():
             "dmc_decode_step_static_scratch": (C.c_int, [vp, i32, vp, vp, vp, vp, vp]),
             "dmc_cache_lengths": (C.c_int, [vp, i32, vp, vp]),
             "dmc_cache_export_heads": (C.c_int, [vp, i32, i32, vp, i32, vp, vp, vp, vp, vp]),
+            "dmc_cache_export_heads_padded": (C.c_int, [vp, i32, i32, vp, i32, vp, vp, vp, vp, vp]),
             "dmc_cache_status": (C.c_int, [vp, vp, C.POINTER(C.c_uint32), C.POINTER(i64)]),
             "dmc_status_string": (C.c_char_p, [C.c_int]),
         }
@@ -145,6 +146,12 @@ def dmc_cache_export_heads(handle, layer, n, head_ids_ptr, cap, k_out_ptr, v_out
                            len_out_ptr, stream) -> int:
     return lib().dmc_cache_export_heads(handle, layer, n, head_ids_ptr, cap, k_out_ptr, v_out_ptr,
                                         z_out_ptr, len_out_ptr, stream)
+
+
+def dmc_cache_export_heads_padded(handle, layer, n, head_ids_ptr, cap, k_out_ptr, v_out_ptr,
+                                  z_out_ptr, len_out_ptr, stream) -> int:
+    return lib().dmc_cache_export_heads_padded(handle, layer, n, head_ids_ptr, cap, k_out_ptr,
+                                               v_out_ptr, z_out_ptr, len_out_ptr, stream)
 
 
 def dmc_cache_status(handle, stream):
@@ -249,12 +256,14 @@ class DmcCache:
         ids = t.as_tensor(head_ids, dtype=t.int32, device=self.device)
         n = ids.numel()
         D = self.cfg.head_dim
-        k = t.zeros((n, cap, D), dtype=self.dtype, device=self.device)
-        v = t.zeros((n, cap, D), dtype=self.dtype, device=self.device)
-        z = t.zeros((n, cap), dtype=t.float32, device=self.device)
-        ln = t.zeros(n, dtype=t.int32, device=self.device)
-        _check(dmc_cache_export_heads(self.handle, layer, n, ids.data_ptr(), cap, k.data_ptr(),
-                                      v.data_ptr(), z.data_ptr(), ln.data_ptr(), self._s(stream)),
+        make = t.empty if n else t.zeros  # padded: every row is written
+        k = make((n, cap, D), dtype=self.dtype, device=self.device)
+        v = make((n, cap, D), dtype=self.dtype, device=self.device)
+        z = make((n, cap), dtype=t.float32, device=self.device)
+        ln = make(n, dtype=t.int32, device=self.device)
+        _check(dmc_cache_export_heads_padded(self.handle, layer, n, ids.data_ptr(), cap,
+                                             k.data_ptr(), v.data_ptr(), z.data_ptr(),
+                                             ln.data_ptr(), self._s(stream)),
                "dmc_cache_export_heads")
         return k, v, z, ln
 
