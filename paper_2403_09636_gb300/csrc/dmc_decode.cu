@@ -33,7 +33,8 @@
 // anything a preceding kernel of another layer writes, so it may overlap the
 // tail of the previous kernel on the stream. The host does not use the
 // attribute when the previous decode launch of the cache was for the same
-// layer.
+// layer. (Using it there too, with the wait at the kernel's very start, saves the
+// GPU 0.7 us per launch of a one-layer cache and costs the host 2.)
 #include <math.h>
 
 #include <mutex>
@@ -106,15 +107,28 @@ constexpr int kPartialStride = D + 4;
 // The last contributor of a split head merges the nc partial states of workers
 // wf..wf+nc-1 in worker order and writes the head's output row. Lane
 // (cg = lane / 8, dg = lane % 8) sums contributors cg, cg + 4, ... over dims
-// [dg * D / 8, (dg + 1) * D / 8), eight contributors' loads in flight per
-// batch; the four contributor groups are then added with shuffles.
-template <typename T, int D>
+// [dg * D / 8, (dg + 1) * D / 8), 4 NR contributors' loads in flight, the first
+// ones together with the maxima; the four contributor groups are then added with
+// shuffles.
+template <typename T, int D, int NR>  // NR: contributors per lane group in flight
 __device__ __noinline__ void combine_partials(const float* partials, int wf, int first_off,
                                                  int nc, int lane, T* orow) {
   constexpr int PS = kPartialStride<D>;
   constexpr int V4 = D / 32;  // float4 per lane per contributor
   const int cg = lane >> 3, dg = lane & 7;
   auto slot = [&](int i) { return 2 * (wf + i) + (i == 0 ? first_off : 0); };
+  // the accumulators of contributors c0 + 4 r + cg
+  float4 v[NR][V4];
+  auto load = [&](int c0) {
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int c = c0 + 4 * r + cg;
+      const float4* p = reinterpret_cast<const float4*>(partials + (size_t)slot(min(c, nc - 1)) * PS + 4) + dg * V4;
+#pragma unroll
+      for (int k = 0; k < V4; ++k) v[r][k] = __ldcg(p + k);
+    }
+  };
+  load(0);  // they do not wait for the maximum
   float2 ml0 = make_float2(-INFINITY, 0.f);
   if (lane < nc) ml0 = __ldcg(reinterpret_cast<const float2*>(partials + (size_t)slot(lane) * PS));
   float Mc = ml0.x;
@@ -134,32 +148,22 @@ __device__ __noinline__ void combine_partials(const float* partials, int wf, int
     const float w = (i < nc && ml.x != -INFINITY) ? exp2f(ml.x - Mc) : 0.f;
     Lc = fmaf(ml.y, w, Lc);
     const int n32 = min(32, nc - i0);
-    for (int c0 = 0; c0 < n32; c0 += 8) {
-      float4 v[2][V4];
-      float wv[2];
+    for (int c0 = 0; c0 < n32; c0 += 4 * NR) {
+      if (i0 + c0 > 0) load(i0 + c0);
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
+      for (int r = 0; r < NR; ++r) {
         const int c = c0 + 4 * r + cg;  // < 32
-        wv[r] = __shfl_sync(0xffffffffu, w, c);
+        const float wv = __shfl_sync(0xffffffffu, w, c);
         if (c < n32) {
-          const float4* p = reinterpret_cast<const float4*>(partials + (size_t)slot(i0 + c) * PS + 4) + dg * V4;
 #pragma unroll
-          for (int k = 0; k < V4; ++k) v[r][k] = __ldcg(p + k);
-        } else {
-          wv[r] = 0.f;
-#pragma unroll
-          for (int k = 0; k < V4; ++k) v[r][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int k = 0; k < V4; ++k) {
+            o[k].x = fmaf(v[r][k].x, wv, o[k].x);
+            o[k].y = fmaf(v[r][k].y, wv, o[k].y);
+            o[k].z = fmaf(v[r][k].z, wv, o[k].z);
+            o[k].w = fmaf(v[r][k].w, wv, o[k].w);
+          }
         }
       }
-#pragma unroll
-      for (int r = 0; r < 2; ++r)
-#pragma unroll
-        for (int k = 0; k < V4; ++k) {
-          o[k].x = fmaf(v[r][k].x, wv[r], o[k].x);
-          o[k].y = fmaf(v[r][k].y, wv[r], o[k].y);
-          o[k].z = fmaf(v[r][k].z, wv[r], o[k].z);
-          o[k].w = fmaf(v[r][k].w, wv[r], o[k].w);
-        }
     }
   }
 #pragma unroll
@@ -236,10 +240,15 @@ dmc_decode_kernel(const DecodeArgs a) {
   // each, spread over the blocks so that every SM takes part. Such a launch is
   // all latency: cutting the list over every warp left empty ranges between
   // the parts, which each finish and merge had to step over (7B shape, batch 1,
-  // ~550 units on 1824 warps: 45.2 us per launch, 13.1 with one unit each).
+  // ~550 units on 1824 warps: 45.2 us per launch, 13.1 with one unit each). If
+  // the first half of the blocks can take them all, the others leave at once, and
+  // the next launch's blocks start its prologue in their place.
   const bool few = Utot < (long long)gridDim.x * NWARP;
+  const int half = ((int)gridDim.x + 1) / 2;
+  const int nblk = few && Utot <= (long long)half * NWARP ? half : (int)gridDim.x;
   const int NW = few ? (int)Utot : (int)gridDim.x * NWARP;
-  const int wid = few ? warp * (int)gridDim.x + (int)blockIdx.x : (int)blockIdx.x * NWARP + warp;
+  const int wid = !few ? (int)blockIdx.x * NWARP + warp
+                       : (int)blockIdx.x < nblk ? warp * nblk + (int)blockIdx.x : NW;
   const int u0 = wid < NW ? (int)range_start(wid, Utot, NW) : 0;
   const int u1 = wid < NW ? (int)range_start(wid + 1, Utot, NW) : 0;
   const int grp = lane >> 3, l8 = lane & 7;
@@ -303,6 +312,17 @@ dmc_decode_kernel(const DecodeArgs a) {
   if (u0 < u1) {
     load_window(u0);
     for (int s = 0; s < kRing - 1; ++s) issue_next();
+    // a lone page unit is not much longer than the ring: the rest of it comes to
+    // L2 before the grid wait is over (7B shape, batch 1: 12.9 -> 11.0 us per launch
+    // with the query row requested together with the gates and the deeper merge)
+    if (few && wrws[0] > 4 * (kRing - 1)) {
+      const char* page = L.pages + (size_t)wpid[0] * L.page_bytes;
+      const int first = 4 * (kRing - 1) * ROW, bytes = wrws[0] * ROW - first;
+      for (int x = lane * 128; x < bytes; x += 32 * 128) {
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(page + first + x));
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(page + kPage * ROW + first + x));
+      }
+    }
   }
 
   // q, k, v and the slots this launch writes are touched only after this point
@@ -336,8 +356,8 @@ dmc_decode_kernel(const DecodeArgs a) {
       }
     };
     int vh = head_of_unit(U, NVH, u0);
-    load_heads(vh);
-    // the query row of the next head, loaded ahead of its use
+    // the query row of the next head, loaded ahead of its use (the first one
+    // together with the gates: one round trip to memory after the grid wait)
     auto q_ptr = [&](int hv) {
       const int bh = hv / Gv, b = bh / L.Hkv, h = bh % L.Hkv, g = hv % Gv;
       return qL + ((size_t)b * L.Hq + (size_t)h * L.G + g) * ROW + l8 * 16;
@@ -345,6 +365,7 @@ dmc_decode_kernel(const DecodeArgs a) {
     uint4 qraw[NCH];
 #pragma unroll
     for (int c = 0; c < NCH; ++c) qraw[c] = __ldg(reinterpret_cast<const uint4*>(q_ptr(vh) + c * 128));
+    load_heads(vh);
 
     const float qscale = 1.4426950408889634f / sqrtf((float)D);  // log2(e) / sqrt(d_h)
     float qf[EPL], acc[EPL];
@@ -672,7 +693,9 @@ dmc_decode_kernel(const DecodeArgs a) {
             // worker wf + i wrote state 2 (wf + i) + 1 if the head starts
             // inside its range (only possible for i = 0), else 2 (wf + i)
             const int first_off = (hu0 > range_start(wf, Utot, NW)) ? 1 : 0;
-            combine_partials<T, D>(partials, wf, first_off, wl - wf + 1, lane, orow);
+            // (7B batch 32 / 16K context: 50.2 / 27.2 us with 2, 50.2 / 26.2 with 3, 51.0 /
+            // 25.3 with 4; the 8-warp shape has no registers for more than 2)
+            combine_partials<T, D, NWARP == kWarpsOne ? 3 : 2>(partials, wf, first_off, wl - wf + 1, lane, orow);
           }
         }
         m = -INFINITY;

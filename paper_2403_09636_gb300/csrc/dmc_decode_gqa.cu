@@ -112,6 +112,16 @@ __device__ __noinline__ void combine_gqa(const float* partials, int wf, int firs
   const size_t PS = (size_t)G * (D + 2);
   const float* row = partials + (size_t)(on ? g : 0) * (D + 2);
   auto state = [&](int i) { return row + (size_t)(2 * (wf + i) + (i == 0 ? first_off : 0)) * PS; };
+  float2 ml[NB], v[NB][V2];
+  auto load = [&](int i0) {
+#pragma unroll
+    for (int b = 0; b < NB; ++b) {
+      const float2* p = reinterpret_cast<const float2*>(state(min(i0 + b, nc - 1)));
+      ml[b] = __ldcg(p);
+#pragma unroll
+      for (int i = 0; i < V2; ++i) v[b][i] = __ldcg(p + 1 + 4 * i + t);
+    }
+  };
   float Mc = -INFINITY;
 #pragma unroll 4
   for (int i = t; i < nc; i += 4) Mc = fmaxf(Mc, __ldcg(state(i)));
@@ -122,17 +132,10 @@ __device__ __noinline__ void combine_gqa(const float* partials, int wf, int firs
 #pragma unroll
   for (int i = 0; i < V2; ++i) o[i] = make_float2(0.f, 0.f);
   for (int i0 = 0; i0 < nc; i0 += NB) {
-    float2 ml[NB], v[NB][V2];
+    load(i0);
 #pragma unroll
     for (int b = 0; b < NB; ++b) {
-      const bool in = i0 + b < nc;
-      const float2* p = reinterpret_cast<const float2*>(state(in ? i0 + b : i0));
-      ml[b] = in ? __ldcg(p) : make_float2(-INFINITY, 0.f);
-#pragma unroll
-      for (int i = 0; i < V2; ++i) v[b][i] = in ? __ldcg(p + 1 + 4 * i + t) : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int b = 0; b < NB; ++b) {
+      if (i0 + b >= nc) break;
       const float w = (ml[b].x == -INFINITY) ? 0.f : exp2f(ml[b].x - Mc);
       Lc = fmaf(ml[b].y, w, Lc);
 #pragma unroll
@@ -327,7 +330,6 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
       }
     };
     int vh = head_of_unit(U, NH, u0);
-    load_heads(vh);
 
     // A fragments of the group's queries: row g = query g (zero for g >= G),
     // q[0] removed. qa[kk][0]: dims kk*16 + 2t, +1; qa[kk][1]: dims + 8.
@@ -342,7 +344,8 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
       }
     };
     uint32_t qa[KT][2], qn[KT][2];
-    load_q(vh, qn);
+    load_q(vh, qn);  // with the gates: one round trip to memory after the grid wait
+    load_heads(vh);
 
     const float qscale = 1.4426950408889634f / sqrtf((float)D);  // log2(e) / sqrt(d_h)
     float o[KT][4];
