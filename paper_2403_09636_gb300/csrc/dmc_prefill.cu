@@ -28,6 +28,11 @@
 namespace dmc {
 
 constexpr int kPlanThreads = 256;
+// k[t, h, 0] that a thread of the plan has in flight. Every one costs its 128-byte
+// line of DRAM (the floor: 40 us of a 7B layer's 47), but a head's block used to
+// wait for each 256 tokens in turn: one 16384-token prompt, plan of 4096 tokens
+// 16 us, now 7.
+constexpr int kPlanLoads = 8;
 constexpr int kScanThreads = 128;
 
 struct PrefillArgs {
@@ -74,20 +79,30 @@ __global__ void __launch_bounds__(kPlanThreads) dmc_prefill_plan_kernel(const Pr
   if (tid == 0) { s_fail = 0; s_nan = 0; }
   __syncthreads();
   const T* kk = reinterpret_cast<const T*>(a.k);
-  for (int base = 0; base < ntok; base += kPlanThreads) {
-    const int i = base + tid;
-    bool opens = false;
-    if (i < ntok) {
-      const size_t t = (size_t)(t0 + i);
-      const float x = Elt<T>::to_f(kk[(t * L.Hkv + h) * D]);
-      if (x != x) s_nan = 1;
-      // alpha = round(sigmoid(k[0])) = [k[0] >= 0]; alpha = 0 opens a slot,
-      // and so does the first token of an empty head.
-      opens = !(x >= 0.f) || (i == 0 && len_old == 0);
-      L.opens[t * L.Hkv + h] = opens ? 1 : 0;
+  for (int base = 0; base < ntok; base += kPlanThreads * kPlanLoads) {
+    T x0[kPlanLoads];
+#pragma unroll
+    for (int u = 0; u < kPlanLoads; ++u) {
+      const int i = base + u * kPlanThreads + tid;
+      if (i < ntok) x0[u] = kk[((size_t)(t0 + i) * L.Hkv + h) * D];
     }
-    const unsigned bal = __ballot_sync(0xffffffffu, opens);
-    if (lane == 0 && base + warp * 32 < ntok) atomicAdd(&cnt[(base + warp * 32) / kPrefillChunk], __popc(bal));
+#pragma unroll
+    for (int u = 0; u < kPlanLoads; ++u) {
+      const int first = base + u * kPlanThreads + warp * 32, i = first + lane;
+      if (first >= ntok) break;  // the whole warp
+      bool opens = false;
+      if (i < ntok) {
+        const size_t t = (size_t)(t0 + i);
+        const float x = Elt<T>::to_f(x0[u]);
+        if (x != x) s_nan = 1;
+        // alpha = round(sigmoid(k[0])) = [k[0] >= 0]; alpha = 0 opens a slot,
+        // and so does the first token of an empty head.
+        opens = !(x >= 0.f) || (i == 0 && len_old == 0);
+        L.opens[t * L.Hkv + h] = opens ? 1 : 0;
+      }
+      const unsigned bal = __ballot_sync(0xffffffffu, opens);
+      if (lane == 0) atomicAdd(&cnt[first / kPrefillChunk], __popc(bal));
+    }
   }
   __syncthreads();
   // exclusive scan of the chunk counts (nch <= max_seqlen / 128 + 1)
@@ -275,6 +290,7 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
   // launched as a programmatic dependent of the plan: what follows reads its
   // outputs (the copies above read only the prompt)
   griddep_wait();
+  griddep_launch_dependents();  // prompt attention may set itself up
 
   const int base = L.plan[(size_t)h * L.plan_stride + chunk_id(t0, c, s)];
   const unsigned char* op = L.opens + h;

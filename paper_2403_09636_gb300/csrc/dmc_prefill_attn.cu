@@ -367,6 +367,8 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
     __syncthreads();
     tc_fence_after();
   }
+  // a programmatic dependent of the scan: what came before reads only cu_seqlens
+  griddep_wait();
   const uint32_t tmem = pa_uniform(sh.tmem);
   const int nitems = sh.pref[a.num_seqs];
   const int parity = *reinterpret_cast<volatile int*>(&L.ctl[a.layer * 4]);
@@ -1077,8 +1079,17 @@ static cudaError_t launch_pa(PrefillAttnArgs a, const void* k, const void* v, cu
     const long long items = tiles * L.Hkv * a.num_seqs;  // an upper bound
     if (items == 0) continue;
     const int grid = (int)(items < sms ? items : sms);  // one CTA per SM: its shared memory and TMEM
-    dmc_prefill_attn_kernel<G><<<grid, kPaThreads, kPaSmem, stream>>>(a, maps);
-    e = cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(kPaThreads);
+    cfg.dynamicSmemBytes = kPaSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    e = cudaLaunchKernelEx(&cfg, dmc_prefill_attn_kernel<G>, a, maps);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
