@@ -31,7 +31,7 @@ constexpr int kPlanThreads = 256;
 // k[t, h, 0] that a thread of the plan has in flight. Every one costs its 128-byte
 // line of DRAM (the floor: 40 us of a 7B layer's 47), but a head's block used to
 // wait for each 256 tokens in turn: one 16384-token prompt, plan of 4096 tokens
-// 16 us, now 7.
+// 16 us, now 9.
 constexpr int kPlanLoads = 8;
 constexpr int kScanThreads = 128;
 
