@@ -639,14 +639,14 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
     auto value = [&](int w, int rv, bool add, bool last) -> bool {
       const uint32_t tS = tmem + w * 128, tO = tmem + 256 + w * 128;
       const uint64_t vd = v_desc + (kv0 + rv * (kPaTileBytes / 16));
-#pragma unroll
+#pragma unroll 1
       for (int hf = 0; hf < 2; ++hf) {
         if (!wait(&sh.p_full[w][hf], v_par >> w & 1)) return false;
         if (pa_elect()) {
           tc_fence_after();
 #pragma unroll
-          for (int kk = hf * (kPaSlots / 32); kk < (hf + 1) * (kPaSlots / 32); ++kk)
-            pa_mma_ts(tO, tS + kk * 8, vd + kk * (2048 / 16), pa_idesc(true), add || kk > 0);
+          for (int kk = 0; kk < kPaSlots / 32; ++kk)
+            pa_mma_ts(tO, tS + (hf * 4 + kk) * 8, vd + (hf * 4 + kk) * (2048 / 16), pa_idesc(true), add || hf || kk > 0);
           if (hf) {
             pa_commit(smem_u32(&sh.o_full[w]));
             if (last) pa_commit(smem_u32(&sh.kv_empty[rv]));
@@ -832,8 +832,16 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
         for (int c0 = 0; c0 < kPaSlots; c0 += 32) pa_ld32(tS + c0, s + c0);
         pa_wait_ld();
         if (!full) {
+          // (only the columns that some row of the warp does not see)
+          const int seen = __reduce_min_sync(0xffffffffu, vis);
 #pragma unroll
-          for (int i = 0; i < kPaSlots; ++i) s[i] = i < vis ? s[i] : -INFINITY;
+          for (int c0 = 0; c0 < kPaSlots; c0 += 32) {
+            if (c0 + 32 <= seen) continue;
+            const int left = min(max(vis - c0, 0), 32);
+            const uint32_t hide = left == 32 ? 0u : 0xffffffffu << left;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) s[c0 + i] = (hide >> i & 1u) ? -INFINITY : s[c0 + i];
+          }
         }
         float mx[4] = {s[0], s[1], s[2], s[3]};
 #pragma unroll
@@ -965,6 +973,7 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
       tc_fence_after();
       const bool carried = __any_sync(0xffffffffu, sg < 0);
       const float cw = sg < 0 ? pw : 0.f;  // weight of the carried value sums
+      const float2 cw2 = make_float2(cw, cw), inv2 = make_float2(inv, inv);
       unsigned char* st = sh.stage[warp];
       // four lanes write 64 bytes of a row, eight rows at a time
       const int row0 = wq * 32 + (lane >> 2);
@@ -980,15 +989,17 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
           for (int i = 0; i < 32; i += 4) {
             const float4 cv = *reinterpret_cast<const float4*>(M.carry + D + c0 + i);
             if (sg < 0) {  // otherwise nothing was carried, and the buffer need not hold numbers
-              o[i] = fmaf(cw, cv.x, o[i]);
-              o[i + 1] = fmaf(cw, cv.y, o[i + 1]);
-              o[i + 2] = fmaf(cw, cv.z, o[i + 2]);
-              o[i + 3] = fmaf(cw, cv.w, o[i + 3]);
+              const float2 x = fma2(cw2, make_float2(cv.x, cv.y), make_float2(o[i], o[i + 1]));
+              const float2 y = fma2(cw2, make_float2(cv.z, cv.w), make_float2(o[i + 2], o[i + 3]));
+              o[i] = x.x; o[i + 1] = x.y; o[i + 2] = y.x; o[i + 3] = y.y;
             }
           }
         }
 #pragma unroll
-        for (int i = 0; i < 32; ++i) o[i] *= inv;
+        for (int i = 0; i < 32; i += 2) {
+          const float2 x = mul2(make_float2(o[i], o[i + 1]), inv2);
+          o[i] = x.x; o[i + 1] = x.y;
+        }
         __syncwarp();  // the stage has been read
 #pragma unroll
         for (int q4 = 0; q4 < 4; ++q4)
