@@ -9,11 +9,11 @@
 // number of pages whatever the spread of head lengths. Warps are independent
 // workers: there is no barrier between them after the prologue.
 //
-// A warp streams its pages in "quads" of 4 slot rows, one row per 8-lane
+// A warp streams its pages in pieces of kRows = 8 slot rows, two rows per 8-lane
 // group, 16 bytes per lane per 128-byte chunk of a row. Each lane copies its
-// own chunks of K and V with cp.async into a private ring of kRing quads in
+// own chunks of K and V with cp.async into a private ring of kRing pieces in
 // shared memory and later reads back exactly the bytes it copied, so the ring
-// needs no synchronisation; kRing - 1 quads are in flight per warp. A head cut
+// needs no synchronisation; kRing - 1 pieces are in flight per warp. A head cut
 // by range boundaries is finished by whichever of its warps arrives last
 // (a counter, no waiting), which merges the partial softmax states in worker
 // order, so results are deterministic.
@@ -47,10 +47,21 @@ namespace dmc {
 // Worker warps per block: a launch over one layer ends with a tail (its last
 // heads finish while other warps idle), which fewer, longer warp ranges make
 // shorter; a launch over several layers pays the tail once, and streams faster
-// with more warps in flight.
+// with more warps in flight. Two rows per lane group and packed fp32 arithmetic
+// (about 170 instructions per 8 rows of a warp instead of 420) let four or five
+// warps keep up with HBM: us per layer-step against 6 / 8 warps with one row, 7B
+// batch 32 49.1 (51.1) with one launch per layer, 49.7 (54.2) with one for four,
+// mixed ratios 74.5 (78.9), head_dim 64 34.5 (38.5), window 12 50.6 (53.4).
 constexpr int kWarpsOne = kDecodeWarpsPerBlock;
 constexpr int kWarpsWalk = kDecodeWalkWarpsPerBlock;
-constexpr int kRing = 5;        // quads per warp ring (kRing - 1 in flight)
+constexpr int kRows = 8;        // slot rows per piece: rows grp and grp + 4 of it are an 8-lane group's
+// Pieces per warp ring (all but one in flight). Measured with 4 / 5 / 6 / 8 warps per
+// block, two blocks per SM, us per launch of the 7B shape at batch 32: ring 3 49.9 /
+// 49.5 / 49.7 / 60.7, ring 4 49.0 / 50.7 / 51.2 / -; over four layers of mixed ratios
+// per layer-step (a whole generation, ms): ring 3 - / 5.97 / 5.99 / 6.03, ring 4 6.06
+// / 6.16 / - / 6.17. Rows of 512 bytes keep ring 3, so that two blocks still fit.
+template <int ROW, int NWARP>
+constexpr int kRing = NWARP == kWarpsOne && ROW < 512 ? 4 : 3;
 constexpr int kWindow = 64;     // page units per warp window (page id + rows to copy)
 constexpr int kHeadWindow = 32; // heads whose gates a warp holds in its lanes
 constexpr int kMaxDecodeBlocks = 512;
@@ -70,20 +81,22 @@ struct DecodeArgs {
   long long q_ls, kv_ls;
 };
 
-template <typename T, int D>
+template <typename T, int D, int NWARP>
 struct DecodeGeom {
   static constexpr int ROW = D * (int)sizeof(T);
+  static constexpr int RING = kRing<ROW, NWARP>;
   static constexpr int NCH = ROW / 128;    // 16-byte chunks per lane of an 8-lane group
   static constexpr int EPC = Chunk<T>::N;  // elements per chunk
   static constexpr int EPL = NCH * EPC;    // elements of a row held by one lane
-  // ring slot of one warp: [2 * NCH chunks][32 lanes][16 bytes], K chunks first
-  static constexpr int WSLOT = 2 * NCH * 32 * 16;
-  static constexpr int WRING = kRing * WSLOT;
+  // ring slot of one warp: [2 row halves][2 * NCH chunks][32 lanes][16 bytes], K chunks first
+  static constexpr int WHALF = 2 * NCH * 32 * 16;
+  static constexpr int WSLOT = 2 * WHALF;
+  static constexpr int WRING = RING * WSLOT;
   static constexpr int WWIN = 2 * kWindow * 4;  // page ids, rows to copy
   static constexpr int WARP_BYTES = WRING + WWIN;
   static constexpr int MISC = 64;
-  static size_t smem_bytes(int nvh, int warps) {
-    return (size_t)warps * WARP_BYTES + MISC + (size_t)(nvh + 1) * 4;
+  static size_t smem_bytes(int nvh) {
+    return (size_t)NWARP * WARP_BYTES + MISC + (size_t)(nvh + 1) * 4;
   }
 };
 
@@ -200,8 +213,9 @@ __device__ __noinline__ void combine_partials(const float* partials, int wf, int
 template <typename T, int D, bool kWin, int NWARP>
 __global__ void __launch_bounds__(NWARP * 32, 2)
 dmc_decode_kernel(const DecodeArgs a) {
-  using G_ = DecodeGeom<T, D>;
+  using G_ = DecodeGeom<T, D, NWARP>;
   using CK = Chunk<T>;
+  constexpr int RING = G_::RING;
   constexpr int ROW = G_::ROW, NCH = G_::NCH, EPC = G_::EPC, EPL = G_::EPL;
   constexpr int PSTRIDE = kPartialStride<D>;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -279,45 +293,49 @@ dmc_decode_kernel(const DecodeArgs a) {
     __syncwarp();
   };
 
-  // issue cursor: unit u0 + ik, quad iq of that unit
-  int ik = 0, iq = 0, inq = -1, islot = 0;
+  // issue cursor: unit u0 + ik, piece iq of the inq of that unit, whose first
+  // row of this lane is at isrc, `irows` rows from the page's end
+  int ik = -1, iq = 0, inq = 0, irows = 0, islot = 0;
+  const char* isrc = nullptr;
   auto issue_next = [&]() {
-    while (ik < n) {
+    while (iq >= inq && ik + 1 < n) {
+      ++ik;
       const int iu = u0 + ik;
       if (iu - pb >= kWindow) load_window(iu);
-      if (inq < 0) inq = (wrws[iu - pb] + 3) >> 2;
-      if (iq < inq) break;
-      ++ik;
+      const int rws = wrws[iu - pb];
       iq = 0;
-      inq = -1;
+      inq = (rws + kRows - 1) / kRows;
+      irows = rws - grp;
+      isrc = L.pages + (size_t)wpid[iu - pb] * L.page_bytes + (size_t)grp * ROW + l8 * 16;
     }
-    if (ik < n) {
-      const int iu = u0 + ik;
-      const int row = iq * 4 + grp;
-      if (row < wrws[iu - pb]) {
-        const char* src = L.pages + (size_t)wpid[iu - pb] * L.page_bytes + (size_t)row * ROW + l8 * 16;
-        const uint32_t dst = ring_s + islot * G_::WSLOT + lane * 16;
+    if (iq < inq) {
+      const uint32_t dst = ring_s + islot * G_::WSLOT + lane * 16;
 #pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-          cp_async16(dst + c * 512, src + c * 128);
-          cp_async16(dst + (NCH + c) * 512, src + (size_t)kPage * ROW + c * 128);
+      for (int x = 0; x < 2; ++x) {
+        if (iq * kRows + 4 * x < irows) {
+          const char* src = isrc + (size_t)(iq * kRows + 4 * x) * ROW;
+#pragma unroll
+          for (int c = 0; c < NCH; ++c) {
+            cp_async16(dst + x * G_::WHALF + c * 512, src + c * 128);
+            cp_async16(dst + x * G_::WHALF + (NCH + c) * 512, src + (size_t)kPage * ROW + c * 128);
+          }
         }
       }
       ++iq;
     }
     cp_async_commit();  // one group per call, possibly empty, on every lane
-    islot = (islot + 1 == kRing) ? 0 : islot + 1;
+    islot = (islot + 1 == RING) ? 0 : islot + 1;
   };
 
   if (u0 < u1) {
     load_window(u0);
-    for (int s = 0; s < kRing - 1; ++s) issue_next();
+    for (int s = 0; s < RING - 1; ++s) issue_next();
     // a lone page unit is not much longer than the ring: the rest of it comes to
     // L2 before the grid wait is over (7B shape, batch 1: 12.9 -> 11.0 us per launch
     // with the query row requested together with the gates and the deeper merge)
-    if (few && wrws[0] > 4 * (kRing - 1)) {
+    if (few && wrws[0] > kRows * (RING - 1)) {
       const char* page = L.pages + (size_t)wpid[0] * L.page_bytes;
-      const int first = 4 * (kRing - 1) * ROW, bytes = wrws[0] * ROW - first;
+      const int first = kRows * (RING - 1) * ROW, bytes = wrws[0] * ROW - first;
       for (int x = lane * 128; x < bytes; x += 32 * 128) {
         asm volatile("prefetch.global.L2 [%0];" ::"l"(page + first + x));
         asm volatile("prefetch.global.L2 [%0];" ::"l"(page + kPage * ROW + first + x));
@@ -407,39 +425,67 @@ dmc_decode_kernel(const DecodeArgs a) {
       if (!owner) {
         const int rows_copied = min(kPage, len_old - j * kPage);
         const int rows = min(kPage, len_old - accum - j * kPage);  // the merged slot is excluded
-        const int nq = (rows_copied + 3) >> 2;
-        for (int qd = 0; qd < nq; ++qd) {
+        const int np = (rows_copied + kRows - 1) / kRows;
+        for (int pc = 0; pc < np; ++pc) {
           issue_next();
-          cp_async_wait<kRing - 1>();  // this lane's copies of quad qd have landed
+          cp_async_wait<RING - 1>();  // this lane's copies of piece pc have landed
           const unsigned char* sl = ring + cslot * G_::WSLOT + lane * 16;
-          cslot = (cslot + 1 == kRing) ? 0 : cslot + 1;
-          float s0 = 0.f, s1 = 0.f;
+          cslot = (cslot + 1 == RING) ? 0 : cslot + 1;
+          float s[2];
 #pragma unroll
-          for (int c = 0; c < NCH; ++c) {
-            float f[EPC];
-            CK::unpack(*reinterpret_cast<const uint4*>(sl + c * 512), f);
+          for (int x = 0; x < 2; ++x) {
+            float2 d = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int e = 0; e < EPC; e += 2) {
-              s0 = fmaf(qf[c * EPC + e], f[e], s0);
-              s1 = fmaf(qf[c * EPC + e + 1], f[e + 1], s1);
+            for (int c = 0; c < NCH; ++c) {
+              float f[EPC];
+              CK::unpack(*reinterpret_cast<const uint4*>(sl + x * G_::WHALF + c * 512), f);
+#pragma unroll
+              for (int e = 0; e < EPC; e += 2)
+                d = fma2(make_float2(qf[c * EPC + e], qf[c * EPC + e + 1]), make_float2(f[e], f[e + 1]), d);
             }
+            s[x] = d.x + d.y;
           }
-          float s = s0 + s1;
-          s += __shfl_xor_sync(0xffffffffu, s, 1);
-          s += __shfl_xor_sync(0xffffffffu, s, 2);
-          s += __shfl_xor_sync(0xffffffffu, s, 4);
-          if (qd * 4 + grp < rows) {
-            const float mn = fmaxf(m, s);
+#pragma unroll
+          for (int off = 1; off < 8; off <<= 1) {
+            s[0] += __shfl_xor_sync(0xffffffffu, s[0], off);
+            s[1] += __shfl_xor_sync(0xffffffffu, s[1], off);
+          }
+          const int left = rows - pc * kRows - grp;  // the group's rows are in it: > 0, > 4
+          if (left > 0) {
+            const bool two = left > 4;
+            const float mn = fmaxf(m, two ? fmaxf(s[0], s[1]) : s[0]);
             const float corr = exp2f(m - mn);
-            const float p = exp2f(s - mn);
-            lsum = fmaf(lsum, corr, p);
+            const float p0 = exp2f(s[0] - mn);
+            lsum = fmaf(lsum, corr, p0);
+            const float2 corr2 = make_float2(corr, corr), p02 = make_float2(p0, p0);
 #pragma unroll
             for (int c = 0; c < NCH; ++c) {
               float f[EPC];
               CK::unpack(*reinterpret_cast<const uint4*>(sl + (NCH + c) * 512), f);
 #pragma unroll
-              for (int e = 0; e < EPC; ++e)
-                acc[c * EPC + e] = fmaf(acc[c * EPC + e], corr, p * f[e]);
+              for (int e = 0; e < EPC; e += 2) {
+                const float2 t = mul2(p02, make_float2(f[e], f[e + 1]));
+                const float2 o = fma2(make_float2(acc[c * EPC + e], acc[c * EPC + e + 1]), corr2, t);
+                acc[c * EPC + e] = o.x;
+                acc[c * EPC + e + 1] = o.y;
+              }
+            }
+            if (two) {
+              const float p1 = exp2f(s[1] - mn);
+              lsum += p1;
+              const float2 p12 = make_float2(p1, p1);
+#pragma unroll
+              for (int c = 0; c < NCH; ++c) {
+                float f[EPC];
+                CK::unpack(*reinterpret_cast<const uint4*>(sl + G_::WHALF + (NCH + c) * 512), f);
+#pragma unroll
+                for (int e = 0; e < EPC; e += 2) {
+                  const float2 o = fma2(p12, make_float2(f[e], f[e + 1]),
+                                        make_float2(acc[c * EPC + e], acc[c * EPC + e + 1]));
+                  acc[c * EPC + e] = o.x;
+                  acc[c * EPC + e + 1] = o.y;
+                }
+              }
             }
             m = mn;
           }
@@ -488,7 +534,7 @@ dmc_decode_kernel(const DecodeArgs a) {
           }
         }
         // When this warp has just streamed the head's last page (unit u - 1),
-        // its last quad holds the old last row in the ring, in the lanes of row
+        // its last piece holds the old last row in the ring, in the lanes of row
         // group (len_old - 1) % 4, and the issue window may still hold that
         // page's id: that group then applies the update without a round trip
         // for either.
@@ -505,7 +551,8 @@ dmc_decode_kernel(const DecodeArgs a) {
                     : ptab[(size_t)bh * L.MPH + (len_old - 1) / kPage];
         }
         const unsigned char* rrow =
-            ring + (size_t)((cslot == 0 ? kRing : cslot) - 1) * G_::WSLOT + lane * 16;
+            ring + (size_t)((cslot == 0 ? RING : cslot) - 1) * G_::WSLOT +
+            ((len_old - 1) >> 2 & 1) * G_::WHALF + lane * 16;
         float zold = 0.f, znew = omega;
         const char* orow = nullptr;
         // window grouping: the slot is the mean of the segment's last W
@@ -693,9 +740,9 @@ dmc_decode_kernel(const DecodeArgs a) {
             // worker wf + i wrote state 2 (wf + i) + 1 if the head starts
             // inside its range (only possible for i = 0), else 2 (wf + i)
             const int first_off = (hu0 > range_start(wf, Utot, NW)) ? 1 : 0;
-            // (7B batch 32 / 16K context: 50.2 / 27.2 us with 2, 50.2 / 26.2 with 3, 51.0 /
-            // 25.3 with 4; the 8-warp shape has no registers for more than 2)
-            combine_partials<T, D, NWARP == kWarpsOne ? 3 : 2>(partials, wf, first_off, wl - wf + 1, lane, orow);
+            // (7B batch 32 / 16K context / four layers of mixed ratios: 49.1 / 24.4 us /
+            // 6.00 ms with 3 per lane group, 49.3 / 23.9 / 6.09 with 4, 49.5 / 23.9 / 6.52 with 6)
+            combine_partials<T, D, 3>(partials, wf, first_off, wl - wf + 1, lane, orow);
           }
         }
         m = -INFINITY;
@@ -744,7 +791,7 @@ dmc_decode_kernel(const DecodeArgs a) {
 // Shared memory and blocks per SM of one warp count (both window variants).
 template <typename T, int D, int NWARP>
 static cudaError_t setup_warps(int nvh, int optin, size_t* smem, int* occ) {
-  *smem = DecodeGeom<T, D>::smem_bytes(nvh, NWARP);
+  *smem = DecodeGeom<T, D, NWARP>::smem_bytes(nvh);
   if (*smem > (size_t)optin) return cudaErrorInvalidConfiguration;
   cudaError_t e = cudaFuncSetAttribute(dmc_decode_kernel<T, D, false, NWARP>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
@@ -770,7 +817,7 @@ static cudaError_t setup_decode(int nvh, DecodePlan* plan) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
-  plan->stages = kRing;
+  plan->stages = DecodeGeom<T, D, kWarpsOne>::RING;
   int occ = 0, occw = 0;
   e = setup_warps<T, D, kWarpsOne>(nvh, optin, &plan->smem, &occ);
   if (e != cudaSuccess) return e;
@@ -850,7 +897,7 @@ cudaError_t decode_launch(const Layout& L, int layer0, int nlayers, int Gv, cons
 // ---------------------------------------------------------------- static scratch
 // Scratch of dmc_decode_step_static_scratch: the split-K partial softmax states
 // of one launch, 8 MiB. That holds two states of head_dim + 4 floats for each
-// of the MHA kernel's 4096 worker warps at most, and the tensor-core kernel's
+// of the MHA kernel's 2560 worker warps at most, and the tensor-core kernel's
 // two states per query of a group of 8 (head_dim + 2 floats each) for up to
 // 252 blocks of 4 warps (a GB300 runs 152). Every GPU that loads the library
 // holds it until exit.

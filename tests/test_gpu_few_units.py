@@ -3,8 +3,8 @@
 Both decode kernels then run fewer workers than the grid has warps. Checked
 against the fp64 oracle at the edges: one head of one slot, heads cut into one
 part per page, and a cache whose unit count crosses the grid's warp count while
-it is decoded (64 heads of 27 pages are 1,792 units, of 28 pages 1,856; a GB300
-runs 1,824 warps of the CUDA-core kernel over one layer). The tolerance is the
+it is decoded (64 heads of 18 pages are 1,216 units, of 19 pages 1,280; a GB300
+runs 1,216 warps of the CUDA-core kernel over one layer, 1,520 over several). The tolerance is the
 dtype's (slots stored in bf16 round at every merge: 2e-2; fp32: 1e-4).
 """
 import pytest
@@ -24,7 +24,8 @@ CASES = [
     _wl("one_head_one_slot", 1, 1, 1, 128, "bf16", (1, 1), 5, 1.0, 71),
     _wl("one_head_f32", 1, 1, 1, 64, "f32", (33, 33), 40, 1.0, 72),
     _wl("mha_b1_long", 1, 4, 4, 128, "bf16", (4000, 4000), 6, 1.0, 73),
-    _wl("mha_crosses_the_warp_count", 8, 8, 8, 128, "bf16", (860, 860), 10, 1.0, 74),
+    _wl("mha_crosses_the_warp_count", 8, 8, 8, 128, "bf16", (572, 572), 10, 1.0, 74),
+    _wl("mha_crosses_the_walk_s_warp_count", 10, 8, 8, 128, "bf16", (572, 572), 10, 1.0, 81),
     _wl("f32_virtual_heads_b1", 1, 6, 2, 128, "f32", (700, 700), 6, 2.0, 75),
     _wl("gqa8_b1_one_slot", 1, 8, 1, 128, "bf16", (1, 1), 5, 1.0, 76),
     _wl("gqa8_b1_long", 1, 16, 2, 128, "bf16", (6000, 6000), 6, 1.0, 77),
