@@ -13,8 +13,8 @@
 //
 // The score fragment (row = query, cols = 2 slots) is exactly the B operand
 // layout of the second product, so P never leaves registers and the output
-// accumulator O^T has no padded rows. K and V move in tiles of 16 slots (half
-// a page): each lane cp.asyncs 16-byte chunks into a per-warp ring in shared
+// accumulator O^T has no padded rows. K and V move in tiles of 32 slots (a
+// page): each lane cp.asyncs 16-byte chunks into a per-warp ring in shared
 // memory, chunks XOR-swizzled by row so that ldmatrix (and ldmatrix.trans for
 // V) reads without bank conflicts; rows past the head's length are
 // zero-filled. The softmax is online in the log2 domain, per query row.
@@ -34,8 +34,15 @@ namespace dmc {
 
 constexpr int kGWarps = kGqaWarpsPerBlock;  // workers per block
 constexpr int kGThreads = kGWarps * 32;
-constexpr int kGRing = 4;     // tiles per warp ring (kGRing - 1 in flight)
-constexpr int kTile = 16;     // slots per tile
+// Tiles per warp ring (all but one in flight): a cache with so many heads that the
+// unit prefixes leave no room for three takes two. A page per softmax step halves
+// the shuffles, exponentials of the running maximum and accumulator rescales of the
+// 16-slot tiles before (70B batch 64: 93.8 -> 90.2 us per launch). Warps x ring,
+// one block per SM: 4 x 3 90.2, 3 x 4 113.1, 5 x 2 91.3, 6 x 2 91.8.
+constexpr int kGRing = 3;
+constexpr int kGRingMany = 2;
+constexpr int kTile = 32;     // slots per tile (a page), worked as two halves of 16
+constexpr int kHalf = 16;
 constexpr int kGWindow = 64;  // page units per warp window
 constexpr int kGMaxBlocks = 256;
 constexpr int kGMaxQueries = 8;
@@ -54,13 +61,13 @@ struct GqaArgs {
   long long q_ls, kv_ls;
 };
 
-template <int D>
+template <int D, int RING>
 struct GqaGeom {
   static constexpr int ROW = D * 2;               // bf16 row bytes
   static constexpr int CPR = ROW / 16;            // 16-byte chunks per row
   static constexpr int KT = D / 16;               // k-steps of S = m-tiles of O^T
-  static constexpr int TILE = 2 * kTile * ROW;    // 16 K rows then 16 V rows
-  static constexpr int WRING = kGRing * TILE;
+  static constexpr int TILE = 2 * kTile * ROW;    // 32 K rows then 32 V rows
+  static constexpr int WRING = RING * TILE;
   static constexpr int WWIN = 2 * kGWindow * 4;   // page ids, rows to copy
   static constexpr int WARP_BYTES = WRING + WWIN;
   static constexpr int MISC = 64;
@@ -153,9 +160,9 @@ __device__ __noinline__ void combine_gqa(const float* partials, int wf, int firs
 }
 
 // kWin: the cache uses the window-grouping approximation (L.window > 0)
-template <int D, bool kWin>
+template <int D, bool kWin, int RING>
 __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaArgs a) {
-  using G_ = GqaGeom<D>;
+  using G_ = GqaGeom<D, RING>;
   constexpr int ROW = G_::ROW, CPR = G_::CPR, KT = G_::KT;
   using CK = Chunk<__nv_bfloat16>;
   extern __shared__ __align__(128) unsigned char smem[];
@@ -276,27 +283,30 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
       if (rws > 0) {
         const char* pg = L.pages + (size_t)wpid[iu - pb] * L.page_bytes;
         const uint32_t dst = ring_s + islot * G_::TILE;
+        // the rows past the head's end are zero-filled up to a half's end; a half
+        // without a row is neither copied nor worked
+        const char* src = pg + (size_t)(lane / CPR) * ROW + (lane % CPR) * 16;
 #pragma unroll
         for (int i = 0; i < 2 * kTile * CPR / 32; ++i) {
-          const int x = lane + 32 * i;
-          const int which = x / (kTile * CPR);  // 0: K, 1: V
-          const int rem = x % (kTile * CPR);
-          const int r = rem / CPR, c = rem % CPR;
-          const int row = it * kTile + r;
-          const bool valid = row < rws;
-          const char* src = pg + (size_t)which * kPage * ROW + (size_t)(valid ? row : 0) * ROW + c * 16;
-          cp_async16_zfill(dst + which * kTile * ROW + swz(r, c, ROW), src, valid);
+          constexpr int RPI = 32 / CPR;  // rows per iteration
+          const int which = i * RPI / kTile, r0 = i * RPI % kTile;  // 0: K, 1: V
+          if (r0 < kHalf || rws > kHalf) {
+            const int r = r0 + lane / CPR;
+            const bool valid = r < rws;
+            cp_async16_zfill(dst + which * kTile * ROW + swz(r, lane % CPR, ROW),
+                             valid ? src + (size_t)which * kPage * ROW + (size_t)r0 * ROW : pg, valid);
+          }
         }
       }
       ++it;
     }
     cp_async_commit();  // one group per call, possibly empty, on every lane
-    islot = (islot + 1 == kGRing) ? 0 : islot + 1;
+    islot = (islot + 1 == RING) ? 0 : islot + 1;
   };
 
   if (n > 0) {
     load_window(u0);
-    for (int s = 0; s < kGRing - 1; ++s) issue_next();
+    for (int s = 0; s < RING - 1; ++s) issue_next();
   }
 
   // q, k, v and the slots this launch writes are touched only after this point
@@ -355,51 +365,66 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
     int len_old = 0, flags = 0, cslot = 0;
     float omega = 0.f;
 
-    // one tile of 16 slots, the first `valid` of them attended
-    auto do_tile = [&](uint32_t tile, int valid) {
-      float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    // one tile of up to 32 slots, the first `valid` of them attended (two: its
+    // second half holds rows)
+    auto do_tile = [&](uint32_t tile, int valid, bool two) {
       const int mi = lane >> 3, r = lane & 7;
       const int srow = (mi >> 1) * 8 + r;
+      float s[8];  // scores of query g at slots 2t, 2t + 1, 8 + 2t, 9 + 2t of each half
 #pragma unroll
-      for (int kk = 0; kk < KT; ++kk) {
-        uint32_t b00, b01, b10, b11;
-        ldmatrix_x4(tile + swz(srow, kk * 2 + (mi & 1), ROW), b00, b01, b10, b11);
-        mma_bf16_16816(sc[0], qa[kk][0], 0u, qa[kk][1], 0u, b00, b01);
-        mma_bf16_16816(sc[1], qa[kk][0], 0u, qa[kk][1], 0u, b10, b11);
+      for (int hf = 0; hf < 2; ++hf) {
+        float sc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+        if (hf == 0 || two) {
+#pragma unroll
+          for (int kk = 0; kk < KT; ++kk) {
+            uint32_t b00, b01, b10, b11;
+            ldmatrix_x4(tile + hf * kHalf * ROW + swz(srow, kk * 2 + (mi & 1), ROW), b00, b01, b10, b11);
+            mma_bf16_16816(sc[0], qa[kk][0], 0u, qa[kk][1], 0u, b00, b01);
+            mma_bf16_16816(sc[1], qa[kk][0], 0u, qa[kk][1], 0u, b10, b11);
+          }
+        }
+        const int left = valid - hf * kHalf - 2 * t;
+        s[4 * hf] = left > 0 ? sc[0][0] * qscale : -INFINITY;
+        s[4 * hf + 1] = left > 1 ? sc[0][1] * qscale : -INFINITY;
+        s[4 * hf + 2] = left > 8 ? sc[1][0] * qscale : -INFINITY;
+        s[4 * hf + 3] = left > 9 ? sc[1][1] * qscale : -INFINITY;
       }
-      // scores of query g at slots 2t, 2t + 1, 8 + 2t, 9 + 2t
-      float s[4] = {sc[0][0] * qscale, sc[0][1] * qscale, sc[1][0] * qscale, sc[1][1] * qscale};
-      if (2 * t >= valid) s[0] = -INFINITY;
-      if (2 * t + 1 >= valid) s[1] = -INFINITY;
-      if (8 + 2 * t >= valid) s[2] = -INFINITY;
-      if (9 + 2 * t >= valid) s[3] = -INFINITY;
-      float mx = fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3]));
+      float mx = fmaxf(fmaxf(fmaxf(s[0], s[1]), fmaxf(s[2], s[3])), fmaxf(fmaxf(s[4], s[5]), fmaxf(s[6], s[7])));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
       const float mn = fmaxf(m, mx);
       const float corr = (m == -INFINITY) ? 0.f : exp2f(m - mn);
-      float p[4];
+      float p[8];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) p[i] = (s[i] == -INFINITY) ? 0.f : exp2f(s[i] - mn);
-      float ps = (p[0] + p[1]) + (p[2] + p[3]);
+      for (int i = 0; i < 8; ++i) p[i] = (s[i] == -INFINITY) ? 0.f : exp2f(s[i] - mn);
+      float ps = ((p[0] + p[1]) + (p[2] + p[3])) + ((p[4] + p[5]) + (p[6] + p[7]));
       ps += __shfl_xor_sync(0xffffffffu, ps, 1);
       ps += __shfl_xor_sync(0xffffffffu, ps, 2);
       lsum = lsum * corr + ps;
       m = mn;
       // output columns of this lane are queries 2t and 2t + 1
-      const float c_lo = __shfl_sync(0xffffffffu, corr, 8 * t);
-      const float c_hi = __shfl_sync(0xffffffffu, corr, 8 * t + 4);
-      const uint32_t pb0 = pack_bf16x2(p[0], p[1]), pb1 = pack_bf16x2(p[2], p[3]);
+      const float2 c2 = make_float2(__shfl_sync(0xffffffffu, corr, 8 * t), __shfl_sync(0xffffffffu, corr, 8 * t + 4));
+      const uint32_t p00 = pack_bf16x2(p[0], p[1]), p01 = pack_bf16x2(p[2], p[3]);
+      const uint32_t p10 = pack_bf16x2(p[4], p[5]), p11 = pack_bf16x2(p[6], p[7]);
       const uint32_t vtile = tile + kTile * ROW;
 #pragma unroll
       for (int mt = 0; mt < KT; ++mt) {
-        o[mt][0] *= c_lo;
-        o[mt][1] *= c_hi;
-        o[mt][2] *= c_lo;
-        o[mt][3] *= c_hi;
+        const float2 lo = mul2(make_float2(o[mt][0], o[mt][1]), c2), hi = mul2(make_float2(o[mt][2], o[mt][3]), c2);
+        o[mt][0] = lo.x;
+        o[mt][1] = lo.y;
+        o[mt][2] = hi.x;
+        o[mt][3] = hi.y;
         uint32_t a0, a1, a2, a3;
         ldmatrix_x4_trans(vtile + swz(srow, mt * 2 + (mi & 1), ROW), a0, a1, a2, a3);
-        mma_bf16_16816(o[mt], a0, a1, a2, a3, pb0, pb1);
+        mma_bf16_16816(o[mt], a0, a1, a2, a3, p00, p01);
+      }
+      if (two) {
+#pragma unroll
+        for (int mt = 0; mt < KT; ++mt) {
+          uint32_t a0, a1, a2, a3;
+          ldmatrix_x4_trans(vtile + kHalf * ROW + swz(srow, mt * 2 + (mi & 1), ROW), a0, a1, a2, a3);
+          mma_bf16_16816(o[mt], a0, a1, a2, a3, p10, p11);
+        }
       }
     };
 
@@ -429,10 +454,10 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
         const int ntl = ceil_div(rows_copied, kTile);
         for (int tl = 0; tl < ntl; ++tl) {
           issue_next();
-          cp_async_wait<kGRing - 1>();
+          cp_async_wait<RING - 1>();
           __syncwarp();  // every lane's copies of this tile have landed
-          do_tile(ring_s + cslot * G_::TILE, max(0, min(kTile, rows - tl * kTile)));
-          cslot = (cslot + 1 == kGRing) ? 0 : cslot + 1;
+          do_tile(ring_s + cslot * G_::TILE, max(0, min(kTile, rows - tl * kTile)), rows_copied - tl * kTile > kHalf);
+          cslot = (cslot + 1 == RING) ? 0 : cslot + 1;
         }
       } else {
         // Algorithm 1 on the KV head's new token, once for the group: lanes
@@ -448,15 +473,15 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
         const bool ring_row = !kWin && accum && k > 0 && j > 0;
         uint4 oraw = make_uint4(0, 0, 0, 0);
         if (ring_row && act) {
-          const int ps = (cslot == 0 ? kGRing : cslot) - 1;
+          const int ps = (cslot == 0 ? RING : cslot) - 1;
           oraw = *reinterpret_cast<const uint4*>(smem + (ring_s - smem_u32(smem)) + ps * G_::TILE +
                                                  (is_v ? kTile * ROW : 0) + swz((len_old - 1) % kTile, c, ROW));
         }
         issue_next();
-        cp_async_wait<kGRing - 1>();
+        cp_async_wait<RING - 1>();
         __syncwarp();  // the reserved tile's slot is free
         const uint32_t tile = ring_s + cslot * G_::TILE;
-        cslot = (cslot + 1 == kGRing) ? 0 : cslot + 1;
+        cslot = (cslot + 1 == RING) ? 0 : cslot + 1;
         int tgt = -1;
         if (accum || len_old % kPage != 0) {
           const int up = u - 1;
@@ -558,14 +583,14 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
         // the new row is row 0 of a one-row tile; the other value rows are
         // zero so that their zero weights give exact zeros
         unsigned char* tp = smem + (tile - smem_u32(smem));
-        for (int x = lane; x < kTile * CPR; x += 32) {
+        for (int x = lane; x < kHalf * CPR; x += 32) {
           const int r = x / CPR, cc = x % CPR;
           *reinterpret_cast<uint4*>(tp + kTile * ROW + swz(r, cc, ROW)) = make_uint4(0, 0, 0, 0);
         }
         __syncwarp();
         if (act) *reinterpret_cast<uint4*>(tp + (is_v ? kTile * ROW : 0) + swz(0, c, ROW)) = nrow;
         __syncwarp();
-        do_tile(tile, 1);
+        do_tile(tile, 1, false);
       }
 
       if (owner || k == n - 1) {
@@ -669,32 +694,41 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
   }  // layers
 }
 
+// Shared memory and blocks per SM with one ring depth (both window variants).
+template <int D, int RING>
+static cudaError_t setup_ring(int nh, int optin, size_t* smem, int* occ) {
+  *smem = GqaGeom<D, RING>::smem_bytes(nh);
+  if (*smem > (size_t)optin) return cudaErrorInvalidConfiguration;
+  cudaError_t e = cudaFuncSetAttribute(dmc_decode_gqa_kernel<D, false, RING>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(dmc_decode_gqa_kernel<D, true, RING>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)*smem);
+  int o = 0, ow = 0;
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, dmc_decode_gqa_kernel<D, false, RING>, kGThreads, *smem);
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ow, dmc_decode_gqa_kernel<D, true, RING>, kGThreads, *smem);
+  if (e != cudaSuccess) return e;
+  *occ = min(o, ow);
+  return *occ < 1 ? cudaErrorInvalidConfiguration : cudaSuccess;
+}
+
 template <int D>
 static cudaError_t setup_gqa(const Layout& L, DecodePlan* plan) {
-  using G_ = GqaGeom<D>;
   int dev = 0, sms = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
+  int occ = 0;
   plan->stages = kGRing;
-  plan->smem = G_::smem_bytes(L.NH);
-  if (plan->smem > (size_t)optin) return cudaErrorInvalidConfiguration;
-  e = cudaFuncSetAttribute(dmc_decode_gqa_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)plan->smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dmc_decode_gqa_kernel<D, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)plan->smem);
+  e = setup_ring<D, kGRing>(L.NH, optin, &plan->smem, &occ);
+  if (e == cudaErrorInvalidConfiguration) {
+    plan->stages = kGRingMany;
+    e = setup_ring<D, kGRingMany>(L.NH, optin, &plan->smem, &occ);
+  }
   if (e != cudaSuccess) return e;
-  int occ = 0, occw = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, dmc_decode_gqa_kernel<D, false>, kGThreads,
-                                                    plan->smem);
-  if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occw, dmc_decode_gqa_kernel<D, true>, kGThreads,
-                                                      plan->smem);
-  occ = min(occ, occw);
-  if (e != cudaSuccess) return e;
-  if (occ < 1) return cudaErrorInvalidConfiguration;
   plan->grid = min(sms * occ, kGMaxBlocks);
   const long long max_units = (long long)L.NH * (L.MPH + 1);
   const long long max_blocks = (max_units + kGWarps - 1) / kGWarps;
@@ -714,6 +748,15 @@ cudaError_t gqa_setup(const Layout& L, DecodePlan* plan) {
   if (L.D == 64) return setup_gqa<64>(L, plan);
   if (L.D == 128) return setup_gqa<128>(L, plan);
   return cudaErrorInvalidValue;
+}
+
+template <int D>
+static cudaError_t launch_gqa(const cudaLaunchConfig_t& cfg, const DecodePlan& plan, const GqaArgs& a) {
+  if (plan.stages == kGRing)
+    return a.lay.window > 0 ? cudaLaunchKernelEx(&cfg, dmc_decode_gqa_kernel<D, true, kGRing>, a)
+                            : cudaLaunchKernelEx(&cfg, dmc_decode_gqa_kernel<D, false, kGRing>, a);
+  return a.lay.window > 0 ? cudaLaunchKernelEx(&cfg, dmc_decode_gqa_kernel<D, true, kGRingMany>, a)
+                          : cudaLaunchKernelEx(&cfg, dmc_decode_gqa_kernel<D, false, kGRingMany>, a);
 }
 
 cudaError_t gqa_launch(const Layout& L, int layer0, int nlayers, const DecodePlan& plan, bool pdl,
@@ -739,11 +782,8 @@ cudaError_t gqa_launch(const Layout& L, int layer0, int nlayers, const DecodePla
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
   cudaError_t e = cudaErrorInvalidValue;
-  const bool win = L.window > 0;
-  if (L.D == 64) e = win ? cudaLaunchKernelEx(&cfg, dmc_decode_gqa_kernel<64, true>, a)
-                         : cudaLaunchKernelEx(&cfg, dmc_decode_gqa_kernel<64, false>, a);
-  if (L.D == 128) e = win ? cudaLaunchKernelEx(&cfg, dmc_decode_gqa_kernel<128, true>, a)
-                          : cudaLaunchKernelEx(&cfg, dmc_decode_gqa_kernel<128, false>, a);
+  if (L.D == 64) e = launch_gqa<64>(cfg, plan, a);
+  if (L.D == 128) e = launch_gqa<128>(cfg, plan, a);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

@@ -42,3 +42,14 @@ def test_few_units_match_the_oracle(cuda_dev, wl, launch):
     assert run.len_ok, run.len_msgs[:5]
     bad = run.compare()
     assert not bad, bad[:10]
+
+
+@pytest.mark.parametrize("launch", ["stream", "layers"])
+def test_many_grouped_heads(cuda_dev, launch):
+    """4,800 KV heads: the unit prefixes take the shared memory of the tensor-core
+    kernel's third tile per warp."""
+    wl = _wl("gqa2_many_heads", 600, 16, 8, 128, "bf16", (1, 70), 3, 2.0, 82)
+    run = H.Run(wl, cuda_dev, H.random_samples(wl, 64, seed=5), launch=launch)
+    assert run.len_ok, run.len_msgs[:5]
+    bad = run.compare()
+    assert not bad, bad[:10]
