@@ -112,7 +112,7 @@ Offsets offsets(const dmc_cache_config* c) {
   o.pending = at; at = align_up(at + pend * 2 * row);
   o.pending_at = at; at = align_up(at + pend * 4);
   o.pending_z = at; at = align_up(at + pend * 4);
-  o.opens = at; at = align_up(at + (size_t)c->max_prefill_tokens * c->num_kv_heads);
+  o.opens = at; at = align_up(at + (size_t)c->num_kv_heads * o.plan_stride * 16);
   o.plan = at; at = align_up(at + (size_t)c->num_kv_heads * o.plan_stride * 4);
   o.carry = at; at = align_up(at + (size_t)o.plan_stride * c->num_kv_heads * (2 * c->head_dim + 1) * 4);
   o.weights = at; at = align_up(at + (size_t)o.plan_stride * c->num_kv_heads * dmc::kPrefillChunk * 4);
@@ -240,7 +240,7 @@ dmc_status dmc_cache_create(const dmc_cache_config* cfg, void* arena_dev, size_t
   const bool cuda_core = !(cfg->dtype == DMC_BF16 && L.G >= 2 && L.G <= 8);
   L.partial_cap = (int)dmc::partial_states_cap(cuda_core, L.G);
   L.partials_layer_stride = (long long)L.partial_cap * (L.D + 4);
-  L.opens = reinterpret_cast<unsigned char*>(base + o.opens);
+  L.opens = reinterpret_cast<uint4*>(base + o.opens);
   L.plan = reinterpret_cast<int*>(base + o.plan);
   L.plan_stride = o.plan_stride;
   c->carry = reinterpret_cast<float*>(base + o.carry);

@@ -46,7 +46,7 @@ struct Layout {
   int partial_cap;
   long long partials_layer_stride;  // floats between layers' partial states (CUDA-core kernel;
                                     // 0: one region shared by all layers)
-  unsigned char* opens;    // [max_prefill_tokens][Hkv]: token opens a slot
+  uint4* opens;            // [Hkv][plan_stride]: 128 bits per prompt chunk, token opens a slot
   int* plan;               // [Hkv][plan_stride]: first slot index per prompt chunk
   int plan_stride;
   int max_prefill_tokens;
@@ -266,11 +266,6 @@ __device__ __forceinline__ void mma_bf16_16816(float* d, uint32_t a0, uint32_t a
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void griddep_launch_dependents() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
-
-// Named barrier over the first `threads` threads of the block.
-__device__ __forceinline__ void named_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 }  // namespace dmc

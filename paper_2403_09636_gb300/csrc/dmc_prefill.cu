@@ -7,7 +7,9 @@
 // omega. Two kernels, no host synchronisation:
 //
 //  plan: one block per (sequence, KV head). Reads k[t, h, 0] of the prompt,
-//        records which tokens open a slot (one byte per token and head), counts
+//        records which tokens open a slot (128 bits per chunk and head: a byte
+//        per token and head, strided, cost plan + scan of a 7B layer 281 us
+//        instead of 272, of one 2048-token prompt 28.7 instead of 24.6), counts
 //        openings per 128-token chunk, takes pages for the head's new slots from
 //        the pool (one atomic per head), and stores each chunk's first slot index.
 //  scan: one block per (128-token chunk, KV head, sequence). The block owns the
@@ -28,11 +30,11 @@
 namespace dmc {
 
 constexpr int kPlanThreads = 256;
-// k[t, h, 0] that a thread of the plan has in flight. Every one costs its 128-byte
-// line of DRAM (the floor: 40 us of a 7B layer's 47), but a head's block used to
-// wait for each 256 tokens in turn: one 16384-token prompt, plan of 4096 tokens
-// 16 us, now 9.
-constexpr int kPlanLoads = 8;
+// Chunks of a warp of the plan in flight, four k[t, h, 0] a lane each. Every one
+// costs its 128-byte line of DRAM (the floor: 40 us of a 7B layer's 47), but a
+// head's block used to wait for each 256 tokens in turn: one 16384-token prompt,
+// plan of 4096 tokens 16 us, now 9.
+constexpr int kPlanChunks = 2;  // 4: the same
 constexpr int kScanThreads = 128;
 
 struct PrefillArgs {
@@ -75,35 +77,45 @@ __global__ void __launch_bounds__(kPlanThreads) dmc_prefill_plan_kernel(const Pr
   const int ntok = t1 - t0;
   const int nch = ceil_div(ntok, kPrefillChunk);
   const int len_old = len[bh];
-  for (int c = tid; c < nch; c += kPlanThreads) cnt[c] = 0;
   if (tid == 0) { s_fail = 0; s_nan = 0; }
   __syncthreads();
   const T* kk = reinterpret_cast<const T*>(a.k);
-  for (int base = 0; base < ntok; base += kPlanThreads * kPlanLoads) {
-    T x0[kPlanLoads];
+  uint4* opens = L.opens + (size_t)h * L.plan_stride + chunk_id(t0, 0, s);  // chunk c: opens[c]
+  bool nan = false;
+  for (int cb = warp; cb < nch; cb += kPlanThreads / 32 * kPlanChunks) {  // a chunk is a warp's
+    T x0[kPlanChunks][4];
 #pragma unroll
-    for (int u = 0; u < kPlanLoads; ++u) {
-      const int i = base + u * kPlanThreads + tid;
-      if (i < ntok) x0[u] = kk[((size_t)(t0 + i) * L.Hkv + h) * D];
-    }
+    for (int u = 0; u < kPlanChunks; ++u)
 #pragma unroll
-    for (int u = 0; u < kPlanLoads; ++u) {
-      const int first = base + u * kPlanThreads + warp * 32, i = first + lane;
-      if (first >= ntok) break;  // the whole warp
-      bool opens = false;
-      if (i < ntok) {
-        const size_t t = (size_t)(t0 + i);
-        const float x = Elt<T>::to_f(x0[u]);
-        if (x != x) s_nan = 1;
-        // alpha = round(sigmoid(k[0])) = [k[0] >= 0]; alpha = 0 opens a slot,
-        // and so does the first token of an empty head.
-        opens = !(x >= 0.f) || (i == 0 && len_old == 0);
-        L.opens[t * L.Hkv + h] = opens ? 1 : 0;
+      for (int v = 0; v < 4; ++v) {
+        const int i = (cb + u * (kPlanThreads / 32)) * kPrefillChunk + v * 32 + lane;
+        if (i < ntok) x0[u][v] = kk[((size_t)(t0 + i) * L.Hkv + h) * D];
       }
-      const unsigned bal = __ballot_sync(0xffffffffu, opens);
-      if (lane == 0) atomicAdd(&cnt[first / kPrefillChunk], __popc(bal));
+#pragma unroll
+    for (int u = 0; u < kPlanChunks; ++u) {
+      const int c = cb + u * (kPlanThreads / 32);
+      if (c >= nch) break;  // the whole warp
+      unsigned bits[4];
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        const int i = c * kPrefillChunk + v * 32 + lane;
+        bool op = false;
+        if (i < ntok) {
+          const float x = Elt<T>::to_f(x0[u][v]);
+          nan |= x != x;
+          // alpha = round(sigmoid(k[0])) = [k[0] >= 0]; alpha = 0 opens a slot,
+          // and so does the first token of an empty head.
+          op = !(x >= 0.f) || (i == 0 && len_old == 0);
+        }
+        bits[v] = __ballot_sync(0xffffffffu, op);
+      }
+      if (lane == 0) {
+        opens[c] = make_uint4(bits[0], bits[1], bits[2], bits[3]);
+        cnt[c] = __popc(bits[0]) + __popc(bits[1]) + __popc(bits[2]) + __popc(bits[3]);
+      }
     }
   }
+  if (nan) s_nan = 1;
   __syncthreads();
   // exclusive scan of the chunk counts (nch <= max_seqlen / 128 + 1)
   const int per = ceil_div(nch, kPlanThreads);
@@ -218,8 +230,9 @@ __device__ __forceinline__ void fill_ring(const PrefillArgs& a, int h, int bh, i
 constexpr int kRing = 8;        // rows in a lane's ring
 // Rows of a segment past its chunk that its group still adds alone, two at a time
 // (7B at 4x: three on average). More are summed by all groups: at CR 32 plan + scan
-// of 32 x 2048 tokens takes 289 us, with one group for any tail 477; at 4x the
-// exchange costs more than it saves (297 us if every tail is shared, 281 so).
+// of 32 x 2048 tokens took 289 us so (281 now), with one group for any tail 477; at
+// 4x the exchange costs more than it saves (297 us if every tail was shared, 281 so,
+// 272 now).
 constexpr int kLongTail = 8;
 constexpr int kRingBatch = 4;   // rows per async-copy group
 constexpr size_t kScanRingBytes = (size_t)kRing * 2 * kScanThreads * 16;
@@ -231,7 +244,7 @@ constexpr size_t kScanRingBytes = (size_t)kRing * 2 * kScanThreads * 16;
 // most one more read of its rows), and one that continues the head's last slot
 // takes the old tokens still inside the window from the head's ring (token p of
 // the segment at entry p % W). With the spill-free 128 registers (4 blocks per SM)
-// plan + scan of a 7B layer (32 x 2048 tokens at 4x, W = 12) takes 380 us; one warp
+// plan + scan of a 7B layer (32 x 2048 tokens at 4x, W = 12) takes 366 us; one warp
 // per segment, rows straight into registers, took 883.
 template <typename T, int D, bool kWin>
 __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_kernel(const PrefillArgs a) {
@@ -293,8 +306,8 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
   griddep_launch_dependents();  // prompt attention may set itself up
 
   const int base = L.plan[(size_t)h * L.plan_stride + chunk_id(t0, c, s)];
-  const unsigned char* op = L.opens + h;
-  const size_t ostride = (size_t)L.Hkv;
+  const int nch = ceil_div(t1 - t0, kPrefillChunk);
+  const uint4* opens = L.opens + (size_t)h * L.plan_stride + chunk_id(t0, c, s);  // [1]: the next chunk's
   const T* qq = reinterpret_cast<const T*>(a.q);
   // omega = sigmoid(q[0]) (group mean for GQA); the group's loads, up to eight
   // at a time, are in flight together
@@ -317,18 +330,18 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
   const int pfirst = max(base - 1, 0) / kPage;
   if (base >= 0 && tid < kMaxPages && pfirst + tid < L.MPH)
     s_page[tid] = L.page_table[((size_t)a.layer * L.NH + bh) * L.MPH + pfirst + tid];
-  // one thread per token: does it open a slot, and its omega; the same for the
-  // next 128 tokens' openings (the first of them ends the chunk's last segment)
+  // the chunk's opening bits and the next one's (the first of those ends the
+  // chunk's last segment); one thread per token: its omega
   {
-    const int t = a0 + tid, tn = a1 + tid;
-    const bool f = t < a1 && op[(size_t)t * ostride];
-    const bool fn = tn < t1 && op[(size_t)tn * ostride];
-    const float w = t < a1 ? omega(t) : 0.f;
+    const unsigned* bits = reinterpret_cast<const unsigned*>(opens);
+    const unsigned mine = bits[warp];
+    unsigned other = 0;
+    if (lane == 0 && c + 1 < nch) other = bits[4 + warp];
+    const float w = a0 + tid < a1 ? omega(a0 + tid) : 0.f;
     s_w[tid] = w;
     if (a.weights != nullptr)
-      a.weights[((size_t)chunk_id(t0, c, s) * L.Hkv + h) * kPrefillChunk + tid] = f ? -w : w;
-    const unsigned bal = __ballot_sync(0xffffffffu, f), nbal = __ballot_sync(0xffffffffu, fn);
-    if (lane == 0) { s_bal[warp] = bal; s_nbal[warp] = nbal; }
+      a.weights[((size_t)chunk_id(t0, c, s) * L.Hkv + h) * kPrefillChunk + tid] = (mine >> lane) & 1u ? -w : w;
+    if (lane == 0) { s_bal[warp] = mine; s_nbal[warp] = other; }
   }
   __syncthreads();
   int nstart = 0, first = -1, next = -1;
@@ -348,11 +361,16 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
   if (next < 0) {  // no opening in the next 128 tokens: search on (uniform)
     if (tid == 0) s_next = t1;
     __syncthreads();
-    for (int b0 = a1 + kPrefillChunk; b0 < t1; b0 += kScanThreads) {
-      const int tt = b0 + tid;
-      const bool gq = tt < t1 && op[(size_t)tt * ostride];
-      if (gq) atomicMin(&s_next, tt);
-      if (__syncthreads_or(gq)) break;
+#pragma unroll 1
+    for (int cb = 2; c + cb < nch; cb += kScanThreads) {
+      bool found = false;
+      if (c + cb + tid < nch) {
+        const uint4 b = opens[cb + tid];
+        const int at = b.x ? __ffs(b.x) : b.y ? 32 + __ffs(b.y) : b.z ? 64 + __ffs(b.z) : b.w ? 96 + __ffs(b.w) : 0;
+        found = at != 0;
+        if (found) atomicMin(&s_next, a0 + (cb + tid) * kPrefillChunk + at - 1);
+      }
+      if (__syncthreads_or(found)) break;
     }
     next = s_next;
   }
@@ -665,9 +683,15 @@ __global__ void __launch_bounds__(kPlanThreads) dmc_prefill_ring_kernel(const Pr
   if (L.plan[(size_t)h * L.plan_stride + chunk_id(t0, 0, s)] < 0) return;  // the plan failed
   if (tid == 0) s_last = -1;
   __syncthreads();
-  for (int b = t1 - kPlanThreads; b + kPlanThreads > t0; b -= kPlanThreads) {
-    const int t = b + tid;
-    if (t >= t0 && L.opens[(size_t)t * L.Hkv + h]) atomicMax(&s_last, t);
+  const int nch = ceil_div(t1 - t0, kPrefillChunk);
+  const uint4* opens = L.opens + (size_t)h * L.plan_stride + chunk_id(t0, 0, s);
+  for (int cb = nch - kPlanThreads; cb + kPlanThreads > 0; cb -= kPlanThreads) {
+    const int c = cb + tid;
+    if (c >= 0) {
+      const uint4 b = opens[c];
+      const int at = b.w ? 127 - __clz(b.w) : b.z ? 95 - __clz(b.z) : b.y ? 63 - __clz(b.y) : b.x ? 31 - __clz(b.x) : -1;
+      if (at >= 0) atomicMax(&s_last, t0 + c * kPrefillChunk + at);
+    }
     if (__syncthreads_or(s_last >= 0)) break;
   }
   const int last = s_last;
