@@ -79,6 +79,7 @@ struct DecodeArgs {
   const char* v;
   char* out;      // at out + i * q_ls: [B][Hq][D]
   long long q_ls, kv_ls;
+  bool overlap;  // launched as a programmatic dependent
 };
 
 template <typename T, int D, int NWARP>
@@ -327,9 +328,24 @@ dmc_decode_kernel(const DecodeArgs a) {
     islot = (islot + 1 == RING) ? 0 : islot + 1;
   };
 
+  int vh = 0, page0 = -1;  // the current head; the last slot's page if the first unit is an owner
   if (u0 < u1) {
     load_window(u0);
     for (int s = 0; s < RING - 1; ++s) issue_next();
+    vh = head_of_unit(U, NVH, u0);
+    const int bh0 = vh / Gv, last0 = len_cur[bh0] - 1;
+    // overlapping the kernel before: an owner unit's old row and z come to L2 before
+    // the grid wait is over (7B shape, us per launch with the new token's rows
+    // requested first: batch 1 10.9 -> 10.5, 4 17.5 -> 16.8, 8 21.6 -> 20.7, 32 49.1 ->
+    // 48.7; without an overlap the look-up costs what it saves)
+    if (a.overlap && U[vh + 1] == u0 + 1 && last0 >= 0) {
+      page0 = ptab[(size_t)bh0 * L.MPH + last0 / kPage];
+      const char* row = L.pages + (size_t)page0 * L.page_bytes + (size_t)(last0 % kPage) * ROW;
+      if (lane < 2 * NCH)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(row + (lane < NCH ? 0 : kPage * ROW) + lane % NCH * 128));
+      else if (lane == 2 * NCH)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(L.z + (size_t)page0 * kPage + last0 % kPage));
+    }
     // a lone page unit is not much longer than the ring: the rest of it comes to
     // L2 before the grid wait is over (7B shape, batch 1: 12.9 -> 11.0 us per launch
     // with the query row requested together with the gates and the deeper merge)
@@ -373,7 +389,6 @@ dmc_decode_kernel(const DecodeArgs a) {
         t_omega = sigmoidf_(qs / (float)L.G);  // omega = sigmoid(mean of the group's q[0])
       }
     };
-    int vh = head_of_unit(U, NVH, u0);
     // the query row of the next head, loaded ahead of its use (the first one
     // together with the gates: one round trip to memory after the grid wait)
     auto q_ptr = [&](int hv) {
@@ -543,12 +558,18 @@ dmc_decode_kernel(const DecodeArgs a) {
         const unsigned gmask = 0xffu << (8 * og);
         if (grp == og) {
         // Algorithm 1 on the new token, in fp32, result rounded to the cache dtype.
+        uint4 kraw[NCH], vraw[NCH];  // requested ahead of the look-up of the last slot
+#pragma unroll
+        for (int c = 0; c < NCH; ++c) {
+          kraw[c] = __ldg(reinterpret_cast<const uint4*>(kL + (size_t)bh * ROW + c * 128 + l8 * 16));
+          vraw[c] = __ldg(reinterpret_cast<const uint4*>(vL + (size_t)bh * ROW + c * 128 + l8 * 16));
+        }
         int tgt = -1;
         if (accum || len_old % kPage != 0) {
           const int up = u - 1;
           tgt = (k > 0 && j > 0 && up >= pb && up - pb < kWindow)
                     ? wpid[up - pb]
-                    : ptab[(size_t)bh * L.MPH + (len_old - 1) / kPage];
+                    : k == 0 && page0 >= 0 ? page0 : ptab[(size_t)bh * L.MPH + (len_old - 1) / kPage];
         }
         const unsigned char* rrow =
             ring + (size_t)((cslot == 0 ? RING : cslot) - 1) * G_::WSLOT +
@@ -571,8 +592,8 @@ dmc_decode_kernel(const DecodeArgs a) {
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
           float kin[EPC], vin[EPC];
-          CK::unpack(__ldg(reinterpret_cast<const uint4*>(kL + (size_t)bh * ROW + c * 128 + l8 * 16)), kin);
-          CK::unpack(__ldg(reinterpret_cast<const uint4*>(vL + (size_t)bh * ROW + c * 128 + l8 * 16)), vin);
+          CK::unpack(kraw[c], kin);
+          CK::unpack(vraw[c], vin);
           if (c == 0 && l8 == 0) kin[0] = 0.f;  // k[0] <- 0 (Algorithm 1)
           float kn[EPC], vn[EPC];
           if (W > 0) {
@@ -880,6 +901,7 @@ cudaError_t decode_launch(const Layout& L, int layer0, int nlayers, int Gv, cons
   a.nlayers = nlayers;
   a.q_ls = (long long)L.B * L.Hq * L.row_bytes;
   a.kv_ls = (long long)L.B * L.Hkv * L.row_bytes;
+  a.overlap = pdl;
   a.Gv = Gv;
   a.q = static_cast<const char*>(q);
   a.k = static_cast<const char*>(k);
