@@ -37,7 +37,7 @@ constexpr int kGThreads = kGWarps * 32;
 // Tiles per warp ring (all but one in flight): a cache with so many heads that the
 // unit prefixes leave no room for three takes two. A page per softmax step halves
 // the shuffles, exponentials of the running maximum and accumulator rescales of the
-// 16-slot tiles before (70B batch 64: 93.8 -> 90.2 us per launch). Warps x ring,
+// 16-slot tiles before (70B batch 64: 93.8 -> 90.2 us per launch, 89.7 now). Warps x ring,
 // one block per SM: 4 x 3 90.2, 3 x 4 113.1, 5 x 2 91.3, 6 x 2 91.8.
 constexpr int kGRing = 3;
 constexpr int kGRingMany = 2;
@@ -59,6 +59,7 @@ struct GqaArgs {
   const char* v;
   char* out;            // at out + i * q_ls: [B][Hq][D]
   long long q_ls, kv_ls;
+  bool overlap;         // launched as a programmatic dependent
 };
 
 template <int D, int RING>
@@ -94,8 +95,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // sqrt(kUnitCost n) contributors; more units than that per worker are only taken
 // when the grid has no more warps. Measured for 64 query heads over 8 KV heads,
 // 2048 tokens at 2x, us per launch at batch 1 / 4: 80.6 / 74.0 with every warp a
-// worker and a serial merge; with the merge below and kUnitCost 1, 3, 8: 20.1 /
-// 23.4, 20.1 / 24.4, 23.8 / 31.3.
+// worker and a serial merge; with the merge below and kUnitCost 1, 2, 3, 5: 18.2 /
+// 21.9, 17.7 / 20.3, 18.4 / 23.2, 21.0 / 26.0.
 constexpr float kUnitCost = 2.f;
 __device__ __forceinline__ int gqa_workers(long long U, int nh, int warps) {
   const float per_head = (float)U / (float)nh;
@@ -304,9 +305,25 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
     islot = (islot + 1 == RING) ? 0 : islot + 1;
   };
 
+  int vh = 0, page0 = -1;  // the current head; the last slot's page if the first unit is an owner
   if (n > 0) {
     load_window(u0);
     for (int s = 0; s < RING - 1; ++s) issue_next();
+    vh = head_of_unit(U, NH, u0);
+    const int last0 = len_cur[vh] - 1;
+    // overlapping the kernel before: an owner unit's old row and z come to L2 before
+    // the grid wait is over (64 query heads over 8, us per launch, with the new row
+    // and z requested before the reserved tile: batch 1 18.3 -> 17.7, 4 21.8 -> 20.3,
+    // 64 90.4 -> 89.7)
+    if (a.overlap && U[vh + 1] == u0 + 1 && last0 >= 0) {
+      page0 = ptab[(size_t)vh * L.MPH + last0 / kPage];
+      const char* row = L.pages + (size_t)page0 * L.page_bytes + (size_t)(last0 % kPage) * ROW;
+      constexpr int NL = ROW / 128;
+      if (lane < 2 * NL)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(row + (lane < NL ? 0 : kPage * ROW) + lane % NL * 128));
+      else if (lane == 2 * NL)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(L.z + (size_t)page0 * kPage + last0 % kPage));
+    }
   }
 
   // q, k, v and the slots this launch writes are touched only after this point
@@ -339,7 +356,6 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
         t_omega = sigmoidf_(qs / (float)G);  // omega = sigmoid(mean of the group's q[0])
       }
     };
-    int vh = head_of_unit(U, NH, u0);
 
     // A fragments of the group's queries: row g = query g (zero for g >= G),
     // q[0] removed. qa[kk][0]: dims kk*16 + 2t, +1; qa[kk][1]: dims + 8.
@@ -477,18 +493,24 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
           oraw = *reinterpret_cast<const uint4*>(smem + (ring_s - smem_u32(smem)) + ps * G_::TILE +
                                                  (is_v ? kTile * ROW : 0) + swz((len_old - 1) % kTile, c, ROW));
         }
+        // the new row, the last slot's page and its z are requested before the wait
+        // for the reserved tile
+        uint4 iraw = make_uint4(0, 0, 0, 0);
+        if (act) iraw = __ldg(reinterpret_cast<const uint4*>((is_v ? vL : kL) + (size_t)vh * ROW + c * 16));
+        int tgt = -1;
+        if (accum || len_old % kPage != 0) {
+          const int up = u - 1;
+          tgt = (k > 0 && j > 0 && up >= pb && up - pb < kGWindow) ? wpid[up - pb]
+                : k == 0 && page0 >= 0 ? page0
+                                       : ptab[(size_t)vh * L.MPH + (len_old - 1) / kPage];
+        }
+        float zold = 0.f;
+        if (!kWin && accum) zold = L.z[(size_t)tgt * kPage + (len_old - 1) % kPage];
         issue_next();
         cp_async_wait<RING - 1>();
         __syncwarp();  // the reserved tile's slot is free
         const uint32_t tile = ring_s + cslot * G_::TILE;
         cslot = (cslot + 1 == RING) ? 0 : cslot + 1;
-        int tgt = -1;
-        if (accum || len_old % kPage != 0) {
-          const int up = u - 1;
-          tgt = (k > 0 && j > 0 && up >= pb && up - pb < kGWindow)
-                    ? wpid[up - pb]
-                    : ptab[(size_t)vh * L.MPH + (len_old - 1) / kPage];
-        }
         // window grouping: the slot is the mean of the segment's last W tokens,
         // the W - 1 before this one being in the head's ring
         const int W = kWin ? L.window : 0;
@@ -496,7 +518,7 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
         int n_old = 0, nwin = 0;  // tokens before this one, of them in the window
         const char* ring = nullptr;
         const float* ring_w = nullptr;
-        float zold = 0.f, znew = omega;
+        float znew = omega;
         if (W > 0) {
           ring = L.ring + ((size_t)layer * NH + vh) * W * 2 * ROW;
           ring_w = L.ring_w + ((size_t)layer * NH + vh) * W;
@@ -506,14 +528,12 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
             for (int e = 0; e < nwin; ++e) znew += ring_w[(n_old - 1 - e) % Wm];
           }
         } else if (accum) {
-          zold = L.z[(size_t)tgt * kPage + (len_old - 1) % kPage];
           znew = zold + omega;
         }
         uint4 nrow = make_uint4(0, 0, 0, 0);
         if (act) {
           float in[8], nw[8];
-          const char* src_in = (is_v ? vL : kL) + (size_t)vh * ROW + c * 16;
-          CK::unpack(__ldg(reinterpret_cast<const uint4*>(src_in)), in);
+          CK::unpack(iraw, in);
           if (!is_v && c == 0) in[0] = 0.f;  // k[0] <- 0 (Algorithm 1)
           if (W > 0) {
 #pragma unroll
@@ -767,6 +787,7 @@ cudaError_t gqa_launch(const Layout& L, int layer0, int nlayers, const DecodePla
   a.nlayers = nlayers;
   a.q_ls = (long long)L.B * L.Hq * L.row_bytes;
   a.kv_ls = (long long)L.B * L.Hkv * L.row_bytes;
+  a.overlap = pdl;
   a.q = static_cast<const char*>(q);
   a.k = static_cast<const char*>(k);
   a.v = static_cast<const char*>(v);
