@@ -40,8 +40,8 @@
 // the S that overwrites its P, and the softmax); short ones by the chain of an
 // item's few steps and by HBM. Measured, us of this kernel against the one before it
 // (one CTA of 8 warps per 128 rows, two per SM, copies by cp.async, softmax and MMA
-// in series; 893 / 3482 / 2726): 7B 4x, 32 x 2048 tokens 503; 70B 2x, 16 x 4096
-// tokens 1833; one 16384-token prompt in four calls ~1520. What mattered, in order:
+// in series; 893 / 3482 / 2726): 7B 4x, 32 x 2048 tokens ~495; 70B 2x, 16 x 4096
+// tokens ~1800; one 16384-token prompt in four calls ~1490. What mattered, in order:
 // softmax and MMA in warps of their own; one lane issuing under elect.sync (under
 // `lane == 0` an MMA took ~100 cycles to issue); no call or wait loop inlined thirty
 // times and few unrolled copies (the twelve warps run five different programs, and at
