@@ -228,11 +228,11 @@ __device__ __forceinline__ void fill_ring(const PrefillArgs& a, int h, int bh, i
 // at each chunk start it runs across), and chunk 0 also finishes the segment
 // that continues the head's existing last slot.
 constexpr int kRing = 8;        // rows in a lane's ring
-// Rows of a segment past its chunk that its group still adds alone, two at a time
-// (7B at 4x: three on average). More are summed by all groups: at CR 32 plan + scan
-// of 32 x 2048 tokens took 289 us so (281 now), with one group for any tail 477; at
-// 4x the exchange costs more than it saves (297 us if every tail was shared, 281 so,
-// 272 now).
+// Rows of a segment past its chunk that its group still adds alone (7B at 4x: three
+// on average). More are summed by all groups: at CR 32 plan + scan of 32 x 2048
+// tokens took 289 us so (270 now), with one group for any tail 477; at 4x the
+// exchange costs more than it saves (297 us if every tail was shared, 281 so, 272
+// now).
 constexpr int kLongTail = 8;
 constexpr int kRingBatch = 4;   // rows per async-copy group
 constexpr size_t kScanRingBytes = (size_t)kRing * 2 * kScanThreads * 16;
@@ -243,11 +243,13 @@ constexpr size_t kScanRingBytes = (size_t)kRing * 2 * kScanThreads * 16;
 // rows are read again when it ends (they are in L2: a longer segment costs at
 // most one more read of its rows), and one that continues the head's last slot
 // takes the old tokens still inside the window from the head's ring (token p of
-// the segment at entry p % W). With the spill-free 128 registers (4 blocks per SM)
-// plan + scan of a 7B layer (32 x 2048 tokens at 4x, W = 12) takes 366 us; one warp
-// per segment, rows straight into registers, took 883.
+// the segment at entry p % W). Those rows are read one at a time: with six blocks per
+// SM, as in the exact kernel, plan + scan of a 7B layer (32 x 2048 tokens at 4x, W =
+// 12) takes 327 us, with four rows in flight and the four blocks that their registers
+// leave 366 (W = 32 at CR 32: 421 and 501); one warp per segment, rows straight into
+// registers, took 883.
 template <typename T, int D, bool kWin>
-__global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_kernel(const PrefillArgs a) {
+__global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const PrefillArgs a) {
   using CK = Chunk<T>;
   constexpr int ROW = D * (int)sizeof(T);
   constexpr int LPR = ROW / 16;               // lanes per row
@@ -398,7 +400,7 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
   };
   auto add_row = [&](const uint4& kr, const uint4& vr, float w) { add_to(ak, av, zs, kr, vr, w); };
   // The chunk's last segment runs on to `next`. Few rows there are its group's
-  // work, two at a time; more are summed by all groups, 128 tokens at a time.
+  // work; more are summed by all groups, 128 tokens at a time.
   const bool long_tail = next - a1 > kLongTail && (!kWin || next - a1 < L.window);
   auto slot_ptr = [&](int slot) {
     const int page = s_page[slot / kPage - pfirst];
@@ -424,20 +426,10 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
     if (te - tb <= W) return;
     reset();
 #pragma unroll 1
-    for (int t = te - W; t < te; t += 4) {
-      uint4 kr[4], vr[4];
-      float w[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (t + u < te) {
-          kr[u] = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)(t + u) * hrow));
-          vr[u] = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)(t + u) * hrow));
-          w[u] = t + u < a1 && t + u >= a0 ? s_w[t + u - a0] : omega(t + u);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (t + u < te) add_row(kr[u], vr[u], w[u]);
+    for (int t = te - W; t < te; ++t) {
+      const uint4 kr = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)t * hrow));
+      const uint4 vr = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)t * hrow));
+      add_row(kr, vr, t < a1 && t >= a0 ? s_w[t - a0] : omega(t));
     }
   };
   auto group_bits = [&](int gg) {  // the opening tokens of group gg's range
@@ -517,14 +509,18 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
     }
     zs += from[2 * D];
   };
-  // adds the rows t0, t0 + step, ... below te
+  // Adds the rows tb, tb + step, ... below te, kAdd of them in flight. Two at a time
+  // in the exact kernel spill more than they hide (plan + scan of 32 x 2048 tokens at
+  // CR 32: 270 us with one, 281 with two; long ragged prompts 596 and 604), one at a
+  // time in the windowed one costs a 7B layer 331 us instead of 327.
+  constexpr int kAdd = kWin ? 2 : 1;
   auto add_rows = [&](float* xk, float* xv, float& xz, int tb, int step, int te) {
 #pragma unroll 1
-    for (int t = tb; t < te; t += 2 * step) {
-      uint4 kr[2], vr[2];
-      float w[2];
+    for (int t = tb; t < te; t += kAdd * step) {
+      uint4 kr[kAdd], vr[kAdd];
+      float w[kAdd];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < kAdd; ++u) {
         if (t + u * step < te) {
           kr[u] = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)(t + u * step) * hrow));
           vr[u] = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)(t + u * step) * hrow));
@@ -532,7 +528,7 @@ __global__ void __launch_bounds__(kScanThreads, kWin ? 4 : 6) dmc_prefill_scan_k
         }
       }
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
+      for (int u = 0; u < kAdd; ++u)
         if (t + u * step < te) add_to(xk, xv, xz, kr[u], vr[u], w[u]);
     }
   };
