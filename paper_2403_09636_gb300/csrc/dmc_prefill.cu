@@ -336,7 +336,10 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   // chunk's last segment); one thread per token: its omega
   {
     const unsigned* bits = reinterpret_cast<const unsigned*>(opens);
-    const unsigned mine = bits[warp];
+    // (the masks and the bound below hold the walk inside the prompt whatever the
+    // words say: sequences of inconsistent cu_seqlens may share a chunk's entry)
+    const int left = a1 - a0 - warp * 32;
+    const unsigned mine = left >= 32 ? bits[warp] : left > 0 ? bits[warp] & ((1u << left) - 1u) : 0u;
     unsigned other = 0;
     if (lane == 0 && c + 1 < nch) other = bits[4 + warp];
     const float w = a0 + tid < a1 ? omega(a0 + tid) : 0.f;
@@ -354,6 +357,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     if (next < 0 && nb) next = a1 + w * 32 + __ffs(nb) - 1;
     nstart += __popc(b);
   }
+  next = min(next, t1);
   const bool pre = (c == 0) && !(s_bal[0] & 1u);  // continues the existing last slot
   if (base < 0 || (nstart == 0 && !pre)) {
     // the plan failed, or every token belongs to an earlier chunk's segment
@@ -690,7 +694,7 @@ __global__ void __launch_bounds__(kPlanThreads) dmc_prefill_ring_kernel(const Pr
     }
     if (__syncthreads_or(s_last >= 0)) break;
   }
-  const int last = s_last;
+  const int last = min(s_last, t1 - 1);  // inside the prompt whatever the words say
   if (tid >= 32) return;
   const int parity = *reinterpret_cast<const volatile int*>(&L.ctl[a.layer * 4]);
   const int n_old = last >= 0 ? 0 : L.seglen[((size_t)a.layer * 2 + parity) * L.NH + bh];
