@@ -47,7 +47,7 @@ struct PrefillArgs {
   const int* cu;
   int total_tokens, max_seqlen;
   float* carry;    // [chunk id][Hkv][2D + 1] (sum w k, sum w v, sum w), or null
-  float* weights;  // with carry: [chunk id][Hkv][128], omega, negative where the token opens a slot
+  float* weights;  // with carry: [chunk id][Hkv][128], omega, its sign bit set where the token opens a slot
 };
 
 __device__ __forceinline__ bool seq_bounds(const PrefillArgs& a, int s, int& t0, int& t1) {
@@ -344,8 +344,9 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     if (lane == 0 && c + 1 < nch) other = bits[4 + warp];
     const float w = a0 + tid < a1 ? omega(a0 + tid) : 0.f;
     s_w[tid] = w;
-    if (a.weights != nullptr)
-      a.weights[((size_t)chunk_id(t0, c, s) * L.Hkv + h) * kPrefillChunk + tid] = (mine >> lane) & 1u ? -w : w;
+    if (a.weights != nullptr)  // the sign set as a bit: that of a negated NaN is unspecified
+      a.weights[((size_t)chunk_id(t0, c, s) * L.Hkv + h) * kPrefillChunk + tid] =
+          __uint_as_float((__float_as_uint(w) & 0x7fffffffu) | ((mine >> lane) & 1u) << 31);
     if (lane == 0) { s_bal[warp] = mine; s_nbal[warp] = other; }
   }
   __syncthreads();

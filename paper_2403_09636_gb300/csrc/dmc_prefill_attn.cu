@@ -110,7 +110,7 @@ struct PrefillAttnArgs {
   const int* cu;
   int total_tokens, max_seqlen;
   const float* carry;    // [chunk id][Hkv][2D + 1]
-  const float* weights;  // [chunk id][Hkv][128]: omega, negative where the token opens a slot
+  const float* weights;  // [chunk id][Hkv][128]: omega, its sign bit set where the token opens a slot
   char* out;           // [total_tokens][Hq][D]
   int seq_base;        // this launch's first sequence within the call (chunk ids count sequences)
 };
