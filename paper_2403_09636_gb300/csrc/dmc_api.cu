@@ -7,6 +7,7 @@
 #include <new>
 
 #include "dmc_internal.cuh"
+#include "dmc_overlap.h"
 
 namespace dmc {
 cudaError_t decode_setup(const Layout& L, int Gv, DecodePlan* plan);
@@ -44,7 +45,7 @@ struct dmc_cache {
   int Gv;
   bool gqa;  // grouped queries on the tensor-core kernel (one worker per KV head)
   dmc::DecodePlan plan;
-  int last_decode_lo, last_decode_hi;  // layers [lo, hi) of the latest kernel if it was a decode, else empty
+  dmc::DecodeOrder order;
   char* meta;  // lengths, ctl, counters, pool top, error: cleared by create / reset
   size_t meta_bytes;
   float* carry;    // segment sums at prompt chunk starts (prompt attention)
@@ -257,7 +258,6 @@ dmc_status dmc_cache_create(const dmc_cache_config* cfg, void* arena_dev, size_t
   // entry of the CUDA-core kernel (G = 1 for MHA).
   c->gqa = dmc::gqa_supported(L);
   c->Gv = c->gqa ? 1 : L.G;
-  c->last_decode_lo = c->last_decode_hi = 0;
   cudaError_t e = cudaGetDevice(&c->device);
   if (e == cudaSuccess) e = c->gqa ? dmc::gqa_setup(L, &c->plan) : dmc::decode_setup(L, c->Gv, &c->plan);
   if (e == cudaSuccess) e = cudaMemsetAsync(c->meta, 0, c->meta_bytes, stream);
@@ -269,18 +269,10 @@ dmc_status dmc_cache_create(const dmc_cache_config* cfg, void* arena_dev, size_t
   return DMC_OK;
 }
 
-// A decode launch may overlap the tail of the kernel before it on the stream
-// (programmatic dependent launch) only if that kernel was this cache's decode
-// of other layers: its prologue reads the first layer's slot counts, page table
-// and pages, which this cache's prefill and decode of that layer write.
-bool use_pdl(dmc_cache* c, int layer0, int nlayers) {
-  const bool pdl = c->last_decode_hi > c->last_decode_lo &&
-                   (layer0 < c->last_decode_lo || layer0 >= c->last_decode_hi);
-  c->last_decode_lo = layer0;
-  c->last_decode_hi = layer0 + nlayers;
-  return pdl;
+// Whether a decode launch may overlap the launch before it (DecodeOrder).
+bool use_pdl(dmc_cache* c, int layer0, int nlayers, cudaStream_t stream) {
+  return c->order.next_decode(layer0, nlayers, stream, stream != cudaStreamPerThread);
 }
-void no_pdl_next(dmc_cache* c) { c->last_decode_lo = c->last_decode_hi = 0; }
 
 dmc_status dmc_cache_destroy(dmc_cache_t cache) {
   delete cache;
@@ -289,7 +281,7 @@ dmc_status dmc_cache_destroy(dmc_cache_t cache) {
 
 dmc_status dmc_cache_reset(dmc_cache_t c, cudaStream_t stream) {
   if (!c) return DMC_ERR_INVALID_ARG;
-  no_pdl_next(c);
+  c->order.other();
   return cuda_status(cudaMemsetAsync(c->meta, 0, c->meta_bytes, stream));
 }
 
@@ -308,7 +300,7 @@ dmc_status dmc_prefill_compress(dmc_cache_t c, int32_t layer, int32_t first_seq,
   if (!q_dev || !k_dev || !v_dev || !cu_seqlens_dev || !aligned16(k_dev) || !aligned16(v_dev))
     return DMC_ERR_INVALID_ARG;
   if (q_token_stride < 0 || q_head_stride < 0) return DMC_ERR_INVALID_ARG;
-  no_pdl_next(c);
+  c->order.other();
   return cuda_status(dmc::prefill_launch(L, layer, first_seq, num_seqs, q_dev, q_token_stride,
                                          q_head_stride, k_dev, v_dev, cu_seqlens_dev, total_tokens,
                                          max_seqlen, nullptr, nullptr, stream));
@@ -331,7 +323,7 @@ dmc_status dmc_prefill_attention(dmc_cache_t c, int32_t layer, int32_t first_seq
   if (!q_dev || !k_dev || !v_dev || !cu_seqlens_dev || !out_dev || !aligned16(q_dev) ||
       !aligned16(k_dev) || !aligned16(v_dev) || !aligned16(out_dev))
     return DMC_ERR_INVALID_ARG;
-  no_pdl_next(c);
+  c->order.other();
   const long long q_tok = (long long)L.Hq * L.D, q_head = L.D;
   cudaError_t e = dmc::prefill_launch(L, layer, first_seq, num_seqs, q_dev, q_tok, q_head, k_dev,
                                       v_dev, cu_seqlens_dev, total_tokens, max_seqlen, c->carry,
@@ -350,7 +342,7 @@ dmc_status dmc_decode_step(dmc_cache_t c, int32_t layer, const void* q_dev, cons
   if (!aligned16(q_dev) || !aligned16(k_dev) || !aligned16(v_dev) || !aligned16(out_dev) ||
       !q_dev || !k_dev || !v_dev || !out_dev)
     return DMC_ERR_INVALID_ARG;
-  const bool pdl = use_pdl(c, layer, 1);
+  const bool pdl = use_pdl(c, layer, 1, stream);
   if (c->gqa)
     return cuda_status(dmc::gqa_launch(L, layer, 1, c->plan, pdl, q_dev, k_dev, v_dev, out_dev, stream));
   return cuda_status(dmc::decode_launch(L, layer, 1, c->Gv, c->plan, pdl, q_dev, k_dev, v_dev,
@@ -367,7 +359,7 @@ dmc_status dmc_decode_step_layers(dmc_cache_t c, int32_t first_layer, int32_t nu
   if (!aligned16(q_dev) || !aligned16(k_dev) || !aligned16(v_dev) || !aligned16(out_dev) ||
       !q_dev || !k_dev || !v_dev || !out_dev)
     return DMC_ERR_INVALID_ARG;
-  const bool pdl = use_pdl(c, first_layer, num_layers);
+  const bool pdl = use_pdl(c, first_layer, num_layers, stream);
   if (c->gqa)
     return cuda_status(dmc::gqa_launch(L, first_layer, num_layers, c->plan, pdl, q_dev, k_dev, v_dev,
                                        out_dev, stream));
@@ -410,7 +402,7 @@ dmc_status dmc_decode_step_static_scratch(dmc_cache_t c, int32_t layer, const vo
   ls.partials = scratch;
   ls.partial_cap = (int)(floats / state_floats);
   ls.partials_layer_stride = 0;  // one layer per launch here
-  const bool pdl = use_pdl(c, layer, 1);
+  const bool pdl = use_pdl(c, layer, 1, stream);
   if (c->gqa)
     return cuda_status(dmc::gqa_launch(ls, layer, 1, plan, pdl, q_dev, k_dev, v_dev, out_dev, stream));
   return cuda_status(dmc::decode_launch(ls, layer, 1, c->Gv, plan, pdl, q_dev, k_dev, v_dev,

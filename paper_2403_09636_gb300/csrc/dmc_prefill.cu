@@ -305,7 +305,9 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   // launched as a programmatic dependent of the plan: what follows reads its
   // outputs (the copies above read only the prompt)
   griddep_wait();
-  griddep_launch_dependents();  // prompt attention may set itself up
+  // Prompt attention may set itself up. (Only when it is what comes next: a decode
+  // launched as a dependent would read this layer's slots while they are written.)
+  if (a.weights != nullptr) griddep_launch_dependents();
 
   const int base = L.plan[(size_t)h * L.plan_stride + chunk_id(t0, c, s)];
   const int nch = ceil_div(t1 - t0, kPrefillChunk);
