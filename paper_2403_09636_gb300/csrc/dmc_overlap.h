@@ -5,7 +5,8 @@ namespace dmc {
 
 // A decode launch may overlap the tail of the kernel before it on its stream
 // (programmatic dependent launch) only if that kernel was this cache's decode of
-// other layers: its prologue reads slot counts, page table and pages, which this
+// other layers, none of this launch's among them: its prologue reads slot counts, page
+// table and pages (the tensor-core kernel those of its first two layers), which this
 // cache's prefill and decode of those layers write. The cache's latest call is known
 // here in host order, so it is the kernel before it on the stream only if it went to
 // the same one; after a call on another stream the kernel before may be anything,
@@ -17,7 +18,7 @@ struct DecodeOrder {
   // A decode of layers [layer0, layer0 + nlayers) comes next: may it overlap?
   // one_stream: the handle stands for one stream (cudaStreamPerThread does not).
   bool next_decode(int layer0, int nlayers, const void* s, bool one_stream) {
-    const bool ok = hi > lo && one_stream && s == stream && (layer0 < lo || layer0 >= hi);
+    const bool ok = hi > lo && one_stream && s == stream && (layer0 + nlayers <= lo || layer0 >= hi);
     lo = layer0;
     hi = layer0 + nlayers;
     stream = s;

@@ -71,3 +71,16 @@ def test_random_sequences_of_single_layers(rule):
     for _ in range(300):
         _check(rule, [(rng.randrange(4), rng.choice((0, 1, 1, 1)), rng.choice((0, 16)), rng.random() < 0.9)
                       for _ in range(20)])
+
+
+def test_ranges_of_layers_have_to_be_apart(rule):
+    """decode(1), then one launch over layers 0 and 1: it may not read layer 1's counts
+    while the first publishes them."""
+    assert rule([(1, 1, 16, 1), (0, 2, 16, 1), (2, 2, 16, 1), (0, 2, 16, 1)]) == [False, False, True, True]
+
+
+def test_random_sequences_of_ranges(rule):
+    rng = random.Random(4)
+    for _ in range(500):
+        _check(rule, [(lambda lo: (lo, rng.choice((0, 1, 1, 2, 3)), rng.choice((0, 16)), rng.random() < 0.9))
+                      (rng.randrange(5)) for _ in range(20)])
