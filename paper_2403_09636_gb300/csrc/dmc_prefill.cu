@@ -310,6 +310,9 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   if (a.weights != nullptr) griddep_launch_dependents();
 
   const int base = L.plan[(size_t)h * L.plan_stride + chunk_id(t0, c, s)];
+  const int* len_both = L.lengths + (size_t)a.layer * 2 * L.NH + bh;  // as the plan left them
+  const int len_0 = len_both[0], len_1 = len_both[L.NH];
+  const int len = *reinterpret_cast<const volatile int*>(&L.ctl[a.layer * 4]) ? len_1 : len_0;
   const int nch = ceil_div(t1 - t0, kPrefillChunk);
   const uint4* opens = L.opens + (size_t)h * L.plan_stride + chunk_id(t0, c, s);  // [1]: the next chunk's
   const T* qq = reinterpret_cast<const T*>(a.q);
@@ -338,8 +341,9 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   // chunk's last segment); one thread per token: its omega
   {
     const unsigned* bits = reinterpret_cast<const unsigned*>(opens);
-    // (the masks and the bound below hold the walk inside the prompt whatever the
-    // words say: sequences of inconsistent cu_seqlens may share a chunk's entry)
+    // (the masks and the bounds below hold the walk inside the prompt, and the slots
+    // inside the head, whatever the words and `base` say: sequences of inconsistent
+    // cu_seqlens may share a chunk's entry)
     const int left = a1 - a0 - warp * 32;
     const unsigned mine = left >= 32 ? bits[warp] : left > 0 ? bits[warp] & ((1u << left) - 1u) : 0u;
     unsigned other = 0;
@@ -361,9 +365,10 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     nstart += __popc(b);
   }
   next = min(next, t1);
-  const bool pre = (c == 0) && !(s_bal[0] & 1u);  // continues the existing last slot
-  if (base < 0 || (nstart == 0 && !pre)) {
-    // the plan failed, or every token belongs to an earlier chunk's segment
+  const bool pre = c == 0 && base > 0 && !(s_bal[0] & 1u);  // continues the existing last slot
+  if (base < 0 || base + nstart > len || (nstart == 0 && !pre)) {
+    // the plan failed (or the entry is another sequence's), or every token belongs
+    // to an earlier chunk's segment
     cp_async_wait<0>();
     return;
   }
