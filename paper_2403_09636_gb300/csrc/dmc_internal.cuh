@@ -213,6 +213,36 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigne
   }
 }
 
+// Between two tries of a warp_wait: whether to give up, because this wait has lasted
+// longer than kWaitLimitNs (the fault bit is then set) or another warp's has.
+// `since`: when the warp began to wait, 0 at first; returns that time, or 0 to give
+// up. Not inlined: thirty copies of it are a fifth of the prompt-attention kernel's
+// code.
+inline __device__ __noinline__ unsigned long long warp_give_up(volatile int* abort, unsigned long long since,
+                                                               unsigned int* err) {
+  const unsigned long long t = globaltimer_ns();
+  if (since == 0) since = t;
+  if (t - since > kWaitLimitNs) {
+    atomicOr(err, DMC_FAULT_WAIT_TIMEOUT);
+    *abort = 1;
+  }
+  return __any_sync(0xffffffffu, *abort != 0) ? 0 : since;
+}
+
+// Waits (a whole warp) for the phase with the given parity to complete. The warps of
+// a block share `abort` (shared memory, 0 at first): a wait that takes longer than
+// kWaitLimitNs sets DMC_FAULT_WAIT_TIMEOUT and raises it, and every wait of the block
+// that is not over at once then returns false.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort, unsigned int* err) {
+  unsigned long long since = 0;
+#pragma unroll 1
+  while (!__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) {
+    since = warp_give_up(abort, since, err);
+    if (since == 0) return false;
+  }
+  return true;
+}
+
 // cp.async (LDGSTS) of 16 bytes, L2 only, into this thread's shared memory.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");

@@ -273,22 +273,6 @@ __device__ __forceinline__ void pa_rescale(uint32_t tO, float corr) {
   }
 }
 
-// Between two tries of a wait (a whole warp): whether to give up, because this
-// wait has lasted longer than kWaitLimitNs (the fault bit is then set) or
-// another warp's has. `since`: when the warp began to wait, 0 at first; returns
-// that time, or 0 to give up. Not inlined: thirty copies of it are a fifth of the
-// kernel's code.
-__device__ __noinline__ unsigned long long pa_give_up(volatile int* abort, unsigned long long since,
-                                                      unsigned int* err) {
-  const unsigned long long t = globaltimer_ns();
-  if (since == 0) since = t;
-  if (t - since > kWaitLimitNs) {
-    atomicOr(err, DMC_FAULT_WAIT_TIMEOUT);
-    *abort = 1;
-  }
-  return __any_sync(0xffffffffu, *abort != 0) ? 0 : since;
-}
-
 template <int G>
 __global__ void __launch_bounds__(kPaThreads, 1)
 dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps maps) {
@@ -373,21 +357,10 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
   const int nitems = sh.pref[a.num_seqs];
   const int parity = *reinterpret_cast<volatile int*>(&L.ctl[a.layer * 4]);
 
-  // Waits (a whole warp) for the phase with the given parity of a barrier. A
-  // wait that takes longer than kWaitLimitNs sets the fault bit and raises
-  // s_abort, and every wait that is not over at once then returns false: the
-  // warps leave their loops, drain and return. No warp waits for another in any
-  // other way until then.
-  auto wait = [&](uint64_t* bar, uint32_t ph) -> bool {
-    const uint32_t b = smem_u32(bar);
-    unsigned long long since = 0;
-#pragma unroll 1
-    while (!__all_sync(0xffffffffu, mbar_try_wait(b, ph))) {
-      since = pa_give_up(s_abort, since, L.error);
-      if (since == 0) return false;
-    }
-    return true;
-  };
+  // Every wait but the drains at the end (warp_wait): when one gives up, the warps
+  // leave their loops, drain and return. No warp waits for another in any other way
+  // until then.
+  auto wait = [&](uint64_t* bar, uint32_t ph) -> bool { return warp_wait(smem_u32(bar), ph, s_abort, L.error); };
   auto arrive_warp = [&](uint64_t* bar) {  // one arrival per warp, after all its lanes
     __syncwarp();
     if (lane == 0) mbar_arrive(smem_u32(bar));
