@@ -76,7 +76,7 @@ bool valid_config(const dmc_cache_config* c) {
 
 // Byte offsets of every region; returns the total size.
 struct Offsets {
-  size_t pages, z, ptab, meta, lengths, ctl, counters, pool_top, error, meta_end, partials,
+  size_t pages, z, ptab, meta, lengths, ctl, counters, pool_top, error, unbounded, meta_end, partials,
       pending, pending_at, pending_z, opens, plan, carry, weights, ring, ring_w, seglen, total;
   int MPH, plan_stride;
 };
@@ -101,6 +101,7 @@ Offsets offsets(const dmc_cache_config* c) {
   o.seglen = at; at = align_up(at + (c->window > 0 ? (size_t)c->num_layers * 2 * NH * 4 : 0));
   o.pool_top = at; at = align_up(at + 8);
   o.error = at; at = align_up(at + 4);
+  o.unbounded = at; at = align_up(at + 4);
   o.meta_end = at;
   // Both decode kernels (the CUDA-core one for every cache but grouped bf16
   // queries of 2 to 8 per KV head, which run on the tensor-core kernel) keep
@@ -237,6 +238,7 @@ dmc_status dmc_cache_create(const dmc_cache_config* cfg, void* arena_dev, size_t
   L.pending_z = reinterpret_cast<float*>(base + o.pending_z);
   L.pool_top = reinterpret_cast<unsigned long long*>(base + o.pool_top);
   L.error = reinterpret_cast<unsigned int*>(base + o.error);
+  L.unbounded = reinterpret_cast<unsigned int*>(base + o.unbounded);
   L.partials = reinterpret_cast<float*>(base + o.partials);
   const bool cuda_core = !(cfg->dtype == DMC_BF16 && L.G >= 2 && L.G <= 8);
   L.partial_cap = (int)dmc::partial_states_cap(cuda_core, L.G);

@@ -42,6 +42,7 @@ struct Layout {
   float* pending_z;        // [L][NH]: their z
   unsigned long long* pool_top;
   unsigned int* error;
+  unsigned int* unbounded; // prompt attention: the call has written a slot whose value is not finite
   float* partials;         // [partial_cap][D + 2]: split-K partial softmax states (m, l, acc)
   int partial_cap;
   long long partials_layer_stride;  // floats between layers' partial states (CUDA-core kernel;

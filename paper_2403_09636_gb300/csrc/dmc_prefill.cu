@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(kPlanThreads) dmc_prefill_plan_kernel(const Pr
   const int bh = (a.first_seq + s) * L.Hkv + h;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   griddep_launch_dependents();  // the scan may start its copies of k and v
+  if (a.weights != nullptr && (blockIdx.x | blockIdx.y | tid) == 0) *L.unbounded = 0;
   const int parity = *reinterpret_cast<volatile int*>(&L.ctl[a.layer * 4]);
   int* len = L.lengths + ((size_t)a.layer * 2 + parity) * L.NH;
   int t0, t1;
@@ -426,6 +427,12 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     for (int e = 0; e < EPC; ++e) {
       kn[e] = ak[e] * iz;
       vn[e] = av[e] * iz;
+    }
+    if (a.weights != nullptr) {  // (a token's infinite or NaN value is its slot's, too)
+      float x = 0.f;
+#pragma unroll
+      for (int e = 0; e < EPC; ++e) x = fmaf(vn[e], 0.f, x);
+      if (x != x) *L.unbounded = 1;
     }
     if (lr == 0) kn[0] = 0.f;
     *reinterpret_cast<uint4*>(kdst) = CK::pack(kn);

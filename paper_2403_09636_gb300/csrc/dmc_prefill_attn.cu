@@ -51,6 +51,7 @@
 // P V of both query tiles before S of both; two MMA warps (they ran in step).
 #include <cuda.h>
 #include <math.h>
+#include <stddef.h>
 
 #include "dmc_internal.cuh"
 
@@ -102,6 +103,8 @@ struct PaShared {
 };
 constexpr int kPaSmem = sizeof(PaShared) + 1024;  // + alignment of the tiles to 1024 bytes
 static_assert(kPaSmem <= 227 * 1024, "one CTA's shared memory");
+static_assert(offsetof(PaShared, stage) % 1024 == 0, "swizzled rows in the stages (pa_value_clipped)");
+static_assert(4 * 32 * kPaStageRow >= 16 * kPaD * 2, "16 rows of V in four warps' stages");
 
 struct PrefillAttnArgs {
   Layout lay;
@@ -271,6 +274,41 @@ __device__ __forceinline__ void pa_rescale(uint32_t tO, float corr) {
     for (int i = 0; i < 32; ++i) u[i] = __float_as_uint(f[i] * corr);
     pa_st32(tO + c0, u);
   }
+}
+
+// O of query tile 0 += P V over the first `sees` rows of V (ring tile rv) alone; its P
+// has been announced. One warp. Query tile 1's later tokens may see more of the tile.
+// Those rows have weight zero in tile 0, but times a value that is infinite or NaN that
+// is not zero, so a call that wrote such a slot comes here. (7B layer call 816 us before
+// there was a way to tell, 825 with it and the scan's look at every slot, 879 with the
+// rows cut off in every call.) Steps of 16 rows; the last one's, if it is cut, are
+// copied, with the rest set to zero, to the
+// stages of tile 0's epilogue, which its warps have left.
+__device__ __noinline__ void pa_value_clipped(PaShared& sh, uint32_t tmem, int rv, int sees, bool add, bool last) {
+  const int lane = threadIdx.x & 31, r0 = sees & ~15;
+  unsigned char* cut = sh.stage[0];
+#pragma unroll 1
+  for (int x = lane; x < 16 * 16 && sees > r0; x += 32) {
+    const int r = x >> 4, j = x & 15;
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (r0 + r < sees)
+      v = *reinterpret_cast<const uint4*>(sh.kv[rv] + (j >> 3) * (kPaRows * 128) + (r0 + r) * 128 + (j & 7) * 16);
+    *reinterpret_cast<uint4*>(cut + (j >> 3) * (16 * 128) + r * 128 + (j & 7) * 16) = v;
+  }
+  fence_async_smem();
+  __syncwarp();
+  if (pa_elect()) {
+    tc_fence_after();
+#pragma unroll 1
+    for (int r = 0; r < sees; r += 16)
+      pa_mma_ts(tmem + 256, tmem + r / 2,
+                r + 16 <= sees ? pa_desc(smem_u32(sh.kv[rv]) + r * 128, kPaRows * 128, 1024)
+                               : pa_desc(smem_u32(cut), 16 * 128, 1024),
+                pa_idesc(true), add || r > 0);
+    pa_commit(smem_u32(&sh.o_full[0]));
+    if (last) pa_commit(smem_u32(&sh.kv_empty[rv]));
+  }
+  __syncwarp();
 }
 
 template <int G>
@@ -601,6 +639,7 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
   } else if (warp == 8) {
     // ---------------------------------------------------------------- tensor cores
     uint32_t n = 0;  // ring tiles passed
+    const bool unbounded = pa_uniform(*reinterpret_cast<volatile unsigned int*>(L.unbounded)) != 0;
     // bit w, for query tile w: the parity of the next S / P V / item, and whether
     // there has been one
     uint32_t s_par = 0, v_par = 0, q_par = 0, s_any = 0, v_any = 0;
@@ -718,7 +757,15 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
               const int unit = raw ? RAW : kPage;
               if (rows < kPaSlots && rows % unit) zero_rows(rv, rows, (rows + unit - 1) / unit * unit);
             }
-            if (!(ok = value(w, rv, acc >> w & 1, own || !(due >> (w + 1))))) break;
+            const int sees = raw ? im.tok + TT - raw_first(im, 0) : im.nvis[0] - (i - 1) * kPaSlots;
+            if (unbounded && w == 0 && due == 3 && !own && sees < kPaSlots) {
+              if (!(ok = wait(&sh.p_full[0][0], v_par & 1) && wait(&sh.p_full[0][1], v_par & 1))) break;
+              pa_value_clipped(sh, tmem, rv, sees, acc & 1, false);
+              v_par ^= 1u;
+              v_any |= 1u;
+            } else if (!(ok = value(w, rv, acc >> w & 1, own || !(due >> (w + 1))))) {
+              break;
+            }
             acc |= 1u << w;
           }
           if (ok && (mask >> w & 1)) {
