@@ -142,6 +142,12 @@ __global__ void lengths_copy_kernel(const Layout L, int layer, int* out) {
 // slots into buffers of 640, 268 MB read and 341 MB written in ~90 us; filling the
 // buffers with zeros and then copying took ~190.
 constexpr int kExportSlots = 64;
+// Blocks of a plain export, what a GB300 holds at once: its heads' lengths are only
+// known on the device, so a block takes every gridDim.y-th piece of a head. (With a
+// block per piece of a head's capacity most had nothing to do: 1024 heads of ~520 slots
+// into buffers of 8192 325 us, 91 so and 93 with one block per head, which takes 1049
+// for 8 heads of 16384 slots, 25 so.)
+constexpr int kExportBlocks = 1216;
 
 template <bool kPad>
 __global__ void __launch_bounds__(256) export_kernel(const Layout L, int layer, const int* ids, int cap, char* kout,
@@ -185,7 +191,8 @@ dmc_status export_heads(dmc_cache_t c, bool pad, int32_t layer, int32_t n, const
     return DMC_ERR_INVALID_ARG;
   // without padding nothing lies beyond the slots a head can hold
   const int slots = pad ? cap : min(cap, c->lay.max_slots);
-  const dim3 grid(n, max(1, min(dmc::ceil_div(slots, kExportSlots), 65535)));
+  const int most = pad ? 65535 : dmc::ceil_div(kExportBlocks, n);
+  const dim3 grid(n, max(1, min(dmc::ceil_div(slots, kExportSlots), most)));
   auto* kernel = pad ? export_kernel<true> : export_kernel<false>;
   kernel<<<grid, 256, 0, stream>>>(c->lay, layer, head_ids_dev, cap, static_cast<char*>(k_out_dev),
                                    static_cast<char*>(v_out_dev), z_out_dev, len_out_dev);
