@@ -215,10 +215,10 @@ __device__ __noinline__ void combine_partials(const float* partials, int wf, int
 // 13 us for every blockDim.x heads: fp32, 4 queries per KV head, d 128, 24 tokens, us
 // per launch at batch 16 / 32 / 48 / 64: 29 / 52 / 72 / 95 so, 21 / 37 / 50 / 67 now.)
 template <int ROW>
-__device__ __noinline__ void write_pending(const Layout& L, const char* pending, const int* pending_at,
+__device__ __noinline__ void write_pending(char* pages, float* z, int nh, const char* pending, const int* pending_at,
                                            const float* pending_z) {
   constexpr int PPH = 2 * ROW / 16, kBatch = 8;  // pieces per head
-  const int pieces = L.NH * PPH;
+  const int pieces = nh * PPH;
   for (int x0 = threadIdx.x; x0 < pieces; x0 += kBatch * blockDim.x) {
     int at[kBatch];
     uint4 row[kBatch];
@@ -235,16 +235,17 @@ __device__ __noinline__ void write_pending(const Layout& L, const char* pending,
     for (int u = 0; u < kBatch; ++u) {
       if (at[u] < 0) continue;
       const int x = x0 + u * blockDim.x, i = x % PPH * 16;
-      char* dst = L.pages + (size_t)(at[u] / kPage) * L.page_bytes + (size_t)(at[u] % kPage) * ROW;
+      char* dst = pages + (size_t)(at[u] / kPage) * (2 * kPage * ROW) + (size_t)(at[u] % kPage) * ROW;
       *reinterpret_cast<uint4*>(dst + (i < ROW ? i : kPage * ROW + i - ROW)) = row[u];
-      if (i == 0) L.z[at[u]] = pending_z[x / PPH];
+      if (i == 0) z[at[u]] = pending_z[x / PPH];
     }
   }
 }
 
 // kWin: the cache uses the window-grouping approximation (L.window > 0);
-// NWARP: worker warps per block
-template <typename T, int D, bool kWin, int NWARP>
+// NWARP: worker warps per block; kVirtual: several virtual heads per KV head (a kernel
+// of its own, since the code that only they need cost the others registers)
+template <typename T, int D, bool kWin, int NWARP, bool kVirtual>
 __global__ void __launch_bounds__(NWARP * 32, 2)
 dmc_decode_kernel(const DecodeArgs a) {
   using G_ = DecodeGeom<T, D, NWARP>;
@@ -255,7 +256,7 @@ dmc_decode_kernel(const DecodeArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
 
   const Layout& L = a.lay;
-  const int Gv = a.Gv;
+  const int Gv = kVirtual ? a.Gv : 1;
   const int NVH = L.NH * Gv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   unsigned char* ring = smem + (size_t)warp * G_::WARP_BYTES;
@@ -818,7 +819,7 @@ dmc_decode_kernel(const DecodeArgs a) {
     // last block of the launch: every owner has finished
     if (Gv > 1) {
       __threadfence();
-      write_pending<ROW>(L, pending, pending_at, pending_z);
+      write_pending<ROW>(L.pages, L.z, L.NH, pending, pending_at, pending_z);
       __syncthreads();
     }
     if (tid == 0) {  // publish the new slot counts
@@ -832,28 +833,28 @@ dmc_decode_kernel(const DecodeArgs a) {
 }
 
 // Shared memory and blocks per SM of one warp count (both window variants).
-template <typename T, int D, int NWARP>
+template <typename T, int D, int NWARP, bool kVirtual>
 static cudaError_t setup_warps(int nvh, int optin, size_t* smem, int* occ) {
   *smem = DecodeGeom<T, D, NWARP>::smem_bytes(nvh);
   if (*smem > (size_t)optin) return cudaErrorInvalidConfiguration;
-  cudaError_t e = cudaFuncSetAttribute(dmc_decode_kernel<T, D, false, NWARP>,
+  cudaError_t e = cudaFuncSetAttribute(dmc_decode_kernel<T, D, false, NWARP, kVirtual>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dmc_decode_kernel<T, D, true, NWARP>,
+    e = cudaFuncSetAttribute(dmc_decode_kernel<T, D, true, NWARP, kVirtual>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
   int o = 0, ow = 0;
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, dmc_decode_kernel<T, D, false, NWARP>, NWARP * 32,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, dmc_decode_kernel<T, D, false, NWARP, kVirtual>, NWARP * 32,
                                                       *smem);
   if (e == cudaSuccess)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ow, dmc_decode_kernel<T, D, true, NWARP>, NWARP * 32,
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ow, dmc_decode_kernel<T, D, true, NWARP, kVirtual>, NWARP * 32,
                                                       *smem);
   if (e != cudaSuccess) return e;
   *occ = min(o, ow);
   return *occ < 1 ? cudaErrorInvalidConfiguration : cudaSuccess;
 }
 
-template <typename T, int D>
+template <typename T, int D, bool kVirtual>
 static cudaError_t setup_decode(int nvh, DecodePlan* plan) {
   int dev = 0, sms = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -862,24 +863,29 @@ static cudaError_t setup_decode(int nvh, DecodePlan* plan) {
   if (e != cudaSuccess) return e;
   plan->stages = DecodeGeom<T, D, kWarpsOne>::RING;
   int occ = 0, occw = 0;
-  e = setup_warps<T, D, kWarpsOne>(nvh, optin, &plan->smem, &occ);
+  e = setup_warps<T, D, kWarpsOne, kVirtual>(nvh, optin, &plan->smem, &occ);
   if (e != cudaSuccess) return e;
   plan->grid = min(sms * occ, kMaxDecodeBlocks);
   // a launch over several layers takes the one-layer shape when its own does
   // not fit (wide rows with many heads)
-  e = setup_warps<T, D, kWarpsWalk>(nvh, optin, &plan->smem_walk, &occw);
+  e = setup_warps<T, D, kWarpsWalk, kVirtual>(nvh, optin, &plan->smem_walk, &occw);
   plan->grid_walk = e == cudaSuccess ? min(sms * occw, kMaxDecodeBlocks) : 0;
   if (e == cudaErrorInvalidConfiguration) e = cudaSuccess;
   return e;
 }
 
+template <typename T, int D>
+static cudaError_t setup_heads(int nvh, int Gv, DecodePlan* plan) {
+  return Gv > 1 ? setup_decode<T, D, true>(nvh, plan) : setup_decode<T, D, false>(nvh, plan);
+}
+
 cudaError_t decode_setup(const Layout& L, int Gv, DecodePlan* plan) {
   const int nvh = L.NH * Gv;
   cudaError_t e = cudaErrorInvalidValue;
-  if (L.esize == 4 && L.D == 64) e = setup_decode<float, 64>(nvh, plan);
-  if (L.esize == 4 && L.D == 128) e = setup_decode<float, 128>(nvh, plan);
-  if (L.esize == 2 && L.D == 64) e = setup_decode<__nv_bfloat16, 64>(nvh, plan);
-  if (L.esize == 2 && L.D == 128) e = setup_decode<__nv_bfloat16, 128>(nvh, plan);
+  if (L.esize == 4 && L.D == 64) e = setup_heads<float, 64>(nvh, Gv, plan);
+  if (L.esize == 4 && L.D == 128) e = setup_heads<float, 128>(nvh, Gv, plan);
+  if (L.esize == 2 && L.D == 64) e = setup_heads<__nv_bfloat16, 64>(nvh, Gv, plan);
+  if (L.esize == 2 && L.D == 128) e = setup_heads<__nv_bfloat16, 128>(nvh, Gv, plan);
   if (e != cudaSuccess) return e;
   // no more warps than the most units a layer can have
   const long long max_units = (long long)nvh * (L.MPH + 1);
@@ -902,8 +908,11 @@ static cudaError_t launch_warps(const DecodeArgs& a, int grid, size_t smem, bool
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  if (a.lay.window > 0) return cudaLaunchKernelEx(&cfg, dmc_decode_kernel<T, D, true, NWARP>, a);
-  return cudaLaunchKernelEx(&cfg, dmc_decode_kernel<T, D, false, NWARP>, a);
+  if (a.Gv > 1)
+    return a.lay.window > 0 ? cudaLaunchKernelEx(&cfg, dmc_decode_kernel<T, D, true, NWARP, true>, a)
+                            : cudaLaunchKernelEx(&cfg, dmc_decode_kernel<T, D, false, NWARP, true>, a);
+  return a.lay.window > 0 ? cudaLaunchKernelEx(&cfg, dmc_decode_kernel<T, D, true, NWARP, false>, a)
+                          : cudaLaunchKernelEx(&cfg, dmc_decode_kernel<T, D, false, NWARP, false>, a);
 }
 
 template <typename T, int D>
