@@ -167,7 +167,7 @@ dmc_status dmc_decode_step(dmc_cache_t cache, int32_t layer, const void* q_dev,
  * reads only that layer's cache and inputs, Algorithm 1 and Eq. attn-softmax
  * per KV head, so the layers are independent). Same slots and lengths for
  * every layer as calling dmc_decode_step on the layers in order, and the same
- * outputs up to the order of the split-K sums: the CUDA-core kernel runs more
+ * outputs up to the order of the split-K sums: the CUDA-core kernel may run more
  * warps per block over several layers than over one, so a head may be split
  * over other warps (outputs are bit-identical when neither grid splits a head,
  * and always for the tensor-core kernel). What it saves is one launch and one
@@ -193,7 +193,8 @@ dmc_status dmc_decode_step_layers(dmc_cache_t cache, int32_t first_layer, int32_
  * file-scope __device__ array of 8 MiB (2,097,152 floats) that every GPU
  * loading the library holds until the process exits. One launch needs
  *   2 * grid * 4 states of head_dim + 4 floats   (CUDA-core kernel: MHA, fp32,
- *                                                 groups above 8), or
+ *                                                 groups above 8; 2 * grid * 6
+ *                                                 for caches of many heads), or
  *   2 * grid * 4 * G states of head_dim + 2 floats (tensor-core kernel: bf16
  *                                                 groups of 2 to 8 queries),
  * grid being the cache's decode grid (at most one or two blocks per SM). Every

@@ -48,10 +48,12 @@ namespace dmc {
 // heads finish while other warps idle), which fewer, longer warp ranges make
 // shorter; a launch over several layers pays the tail once, and streams faster
 // with more warps in flight. Two rows per lane group and packed fp32 arithmetic
-// (about 170 instructions per 8 rows of a warp instead of 420) let four or five
-// warps keep up with HBM: us per layer-step against 6 / 8 warps with one row, 7B
-// batch 32 49.1 (51.1) with one launch per layer, 49.7 (54.2) with one for four,
-// mixed ratios 74.5 (78.9), head_dim 64 34.5 (38.5), window 12 50.6 (53.4).
+// (about 170 instructions per 8 rows of a warp instead of 420) let four warps keep up
+// with HBM: us per launch against 6 warps with one row, 7B batch 32 49.1 (51.1),
+// head_dim 64 34.5 (38.5), window 12 50.6 (53.4). Over several layers six (against 8
+// with one row; five are as fast on long heads, but 2560 heads of 24 slots took 25.6 us
+// a layer with five, 17.6 with six and 21.5 with the eight before): 4 layers of mixed
+// ratios 5.99 ms a generation with six, 5.97 with five.
 constexpr int kWarpsOne = kDecodeWarpsPerBlock;
 constexpr int kWarpsWalk = kDecodeWalkWarpsPerBlock;
 constexpr int kRows = 8;        // slot rows per piece: rows grp and grp + 4 of it are an 8-lane group's
@@ -862,6 +864,7 @@ static cudaError_t setup_decode(int nvh, DecodePlan* plan) {
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   plan->stages = DecodeGeom<T, D, kWarpsOne>::RING;
+  plan->warps = kWarpsOne;
   int occ = 0, occw = 0;
   e = setup_warps<T, D, kWarpsOne, kVirtual>(nvh, optin, &plan->smem, &occ);
   if (e != cudaSuccess) return e;
@@ -871,6 +874,17 @@ static cudaError_t setup_decode(int nvh, DecodePlan* plan) {
   e = setup_warps<T, D, kWarpsWalk, kVirtual>(nvh, optin, &plan->smem_walk, &occw);
   plan->grid_walk = e == cudaSuccess ? min(sms * occw, kMaxDecodeBlocks) : 0;
   if (e == cudaErrorInvalidConfiguration) e = cudaSuccess;
+  // With more than 3 heads for every 2 warps a layer of short heads is a chain of owner
+  // updates on each warp, and takes the shape with more warps (bf16 d 128, 24 slots, us
+  // per launch with 4 / 6 warps: 1536 heads 16.2 / 17.8, 1792 16.6 / 16.4, 2048 21.9 /
+  // 16.9, 4096 41.5 / 25.1, 8192 73.4 / 40.8; of ~520 slots: 1024 heads 48.8 / 49.5,
+  // 1536 69.5 / 70.3, 2048 90.9 / 90.6). Lengths are not known on the host.
+  if (plan->grid_walk > 0 && (long long)nvh * 2 > (long long)plan->grid * kWarpsOne * 3) {
+    plan->grid = plan->grid_walk;
+    plan->smem = plan->smem_walk;
+    plan->warps = kWarpsWalk;
+    plan->stages = DecodeGeom<T, D, kWarpsWalk>::RING;
+  }
   return e;
 }
 
@@ -889,9 +903,9 @@ cudaError_t decode_setup(const Layout& L, int Gv, DecodePlan* plan) {
   if (e != cudaSuccess) return e;
   // no more warps than the most units a layer can have
   const long long max_units = (long long)nvh * (L.MPH + 1);
-  plan->grid = (int)std::min<long long>(plan->grid, (max_units + kWarpsOne - 1) / kWarpsOne);
+  plan->grid = (int)std::min<long long>(plan->grid, (max_units + plan->warps - 1) / plan->warps);
   plan->grid_walk = (int)std::min<long long>(plan->grid_walk, (max_units + kWarpsWalk - 1) / kWarpsWalk);
-  plan->partial_states = 2 * max(plan->grid * kWarpsOne, plan->grid_walk * kWarpsWalk);
+  plan->partial_states = 2 * max(plan->grid * plan->warps, plan->grid_walk * kWarpsWalk);
   if (plan->partial_states > L.partial_cap) return cudaErrorInvalidConfiguration;
   return cudaSuccess;
 }
@@ -920,6 +934,7 @@ static cudaError_t launch_decode(const DecodeArgs& a, const DecodePlan& plan, bo
                                  cudaStream_t stream) {
   if (a.nlayers > 1 && plan.grid_walk > 0)
     return launch_warps<T, D, kWarpsWalk>(a, plan.grid_walk, plan.smem_walk, pdl, stream);
+  if (plan.warps == kWarpsWalk) return launch_warps<T, D, kWarpsWalk>(a, plan.grid, plan.smem, pdl, stream);
   return launch_warps<T, D, kWarpsOne>(a, plan.grid, plan.smem, pdl, stream);
 }
 
@@ -950,7 +965,7 @@ cudaError_t decode_launch(const Layout& L, int layer0, int nlayers, int Gv, cons
 // ---------------------------------------------------------------- static scratch
 // Scratch of dmc_decode_step_static_scratch: the split-K partial softmax states
 // of one launch, 8 MiB. That holds two states of head_dim + 4 floats for each
-// of the MHA kernel's 2560 worker warps at most, and the tensor-core kernel's
+// of the MHA kernel's 3072 worker warps at most, and the tensor-core kernel's
 // two states per query of a group of 8 (head_dim + 2 floats each) for up to
 // 252 blocks of 4 warps (a GB300 runs 152). Every GPU that loads the library
 // holds it until exit.

@@ -743,6 +743,7 @@ static cudaError_t setup_gqa(const Layout& L, DecodePlan* plan) {
   if (e != cudaSuccess) return e;
   int occ = 0;
   plan->stages = kGRing;
+  plan->warps = kGWarps;
   e = setup_ring<D, kGRing>(L.NH, optin, &plan->smem, &occ);
   if (e == cudaErrorInvalidConfiguration) {
     plan->stages = kGRingMany;

@@ -14,10 +14,10 @@ constexpr int kPrefillChunk = 128;     // prompt tokens per prefill block
 constexpr int kMaxVirtualHeads = 16384;
 constexpr int kMaxWindow = 32;         // longest window of the window-grouping approximation
 constexpr int kDecodeWarpsPerBlock = 4;      // worker warps per block, CUDA-core decode kernel
-constexpr int kDecodeWalkWarpsPerBlock = 5;  // the same, for a launch over several layers
+constexpr int kDecodeWalkWarpsPerBlock = 6;  // the same, for a launch over several layers or many heads
 constexpr int kGqaWarpsPerBlock = 4;         // worker warps per block, tensor-core decode kernel
 // split-K partial states per layer a cache holds for the decode kernels: two
-// per worker warp of the largest grid (CUDA-core kernel: 512 blocks of up to 5 warps;
+// per worker warp of the largest grid (CUDA-core kernel: 512 blocks of up to 6 warps;
 // tensor-core kernel: 256 blocks x 4 warps, times the group's queries)
 constexpr int kMaxWorkerStates = 8192;
 constexpr int kGqaWorkerStates = 2048;
@@ -63,6 +63,7 @@ __host__ __device__ inline int ceil_div(int a, int b) { return (a + b - 1) / b; 
 // Launch shape of the decode kernel for one cache, fixed at create time.
 struct DecodePlan {
   int grid;            // blocks of a launch over one layer
+  int warps;           // and its worker warps per block
   int stages;          // shared-memory ring depth (pieces or tiles per warp)
   int partial_states;  // split-K partial states one launch may write
   size_t smem;         // dynamic shared memory per block
