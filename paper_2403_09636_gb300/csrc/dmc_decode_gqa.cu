@@ -96,11 +96,14 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // when the grid has no more warps. Measured for 64 query heads over 8 KV heads,
 // 2048 tokens at 2x, us per launch at batch 1 / 4: 80.6 / 74.0 with every warp a
 // worker and a serial merge; with the merge below and kUnitCost 1, 2, 3, 5: 18.2 /
-// 21.9, 17.7 / 20.3, 18.4 / 23.2, 21.0 / 26.0.
+// 21.9, 17.7 / 20.3, 18.4 / 23.2, 21.0 / 26.0. Below two units per worker it is one: 1.2,
+// say, made two of some and one of the others (16 query heads over 8, d 64, batch 16,
+// 40-64 slots: 13 us per launch, 8.5-9 with one unit each, 11-12 with every warp a worker
+// and the serial merge).
 constexpr float kUnitCost = 2.f;
 __device__ __forceinline__ int gqa_workers(long long U, int nh, int warps) {
   const float per_head = (float)U / (float)nh;
-  const float per_worker = fmaxf(1.f, sqrtf(per_head * (1.f / kUnitCost)));
+  const float best = sqrtf(per_head * (1.f / kUnitCost)), per_worker = best < 2.f ? 1.f : best;
   const int want = max(1, (int)((float)U / per_worker));
   return (int)min((long long)min(want, warps), U);
 }
