@@ -238,17 +238,14 @@ constexpr int kLongTail = 8;
 constexpr int kRingBatch = 4;   // rows per async-copy group
 constexpr size_t kScanRingBytes = (size_t)kRing * 2 * kScanThreads * 16;
 
-//
-// Window grouping (kWin): a slot counts only its segment's last W tokens. A
-// segment of at most W tokens is summed as above; of a longer one the last W
-// rows are read again when it ends (they are in L2: a longer segment costs at
-// most one more read of its rows), and one that continues the head's last slot
-// takes the old tokens still inside the window from the head's ring (token p of
-// the segment at entry p % W). Those rows are read one at a time: with six blocks per
-// SM, as in the exact kernel, plan + scan of a 7B layer (32 x 2048 tokens at 4x, W =
-// 12) takes 327 us, with four rows in flight and the four blocks that their registers
-// leave 366 (W = 32 at CR 32: 421 and 501); one warp per segment, rows straight into
-// registers, took 883.
+// Window grouping (kWin): a slot counts only its segment's last W tokens, so the
+// other tokens' rows are neither copied nor added, and a segment that continues the
+// head's last slot takes the old tokens still inside the window from the head's ring
+// (token p of the segment at entry p % W). The copies start once the decisions are
+// known. Plan + scan of 16 x 1500 tokens in us (with every row of a longer segment read,
+// its last W again; and with a warp per segment before that): bf16 d 128, W = 12, CR 4
+// 118 (134; 349), CR 32 99 (125; 143), fp32 d 128 CR 32 112 (189; 165); a 7B layer at
+// 4x, W = 12 284 (323; 891).
 template <typename T, int D, bool kWin>
 __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const PrefillArgs a) {
   using CK = Chunk<T>;
@@ -266,7 +263,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   static_assert((size_t)2 * NG * HS * sizeof(float) <= kScanRingBytes, "heads and tails fit the ring");
   __shared__ __align__(16) unsigned char ring[kScanRingBytes];  // [kRing][K, V][thread] 16 B
   __shared__ float s_w[kPrefillChunk];
-  __shared__ unsigned s_bal[kPrefillChunk / 32], s_nbal[kPrefillChunk / 32];
+  __shared__ unsigned s_bal[2 * kPrefillChunk / 32];  // opening bits: the chunk's, the next one's
   __shared__ int s_page[kMaxPages];
   __shared__ int s_next;
   const Layout& L = a.lay;
@@ -289,11 +286,12 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   const char* vb = a.v + (size_t)h * ROW + lr * 16;
   const uint32_t rbase = smem_u32(ring) + tid * 16;
   auto rk = [&](int pos) { return rbase + (uint32_t)(pos * 2) * kScanThreads * 16; };
+  unsigned counts = 0;  // window grouping: the group's tokens that are summed
   auto issue = [&](int b) {  // copy group b: the group's rows g0 + 4b ... (always committed)
 #pragma unroll
     for (int u = 0; u < kRingBatch; ++u) {
       const int t = g0 + b * kRingBatch + u;
-      if (b < NB && t < g1) {
+      if (b < NB && t < g1 && (!kWin || (counts >> (t - g0) & 1u))) {
         const uint32_t dk = rk((b % 2) * kRingBatch + u);
         cp_async16(dk, kb + (size_t)t * hrow);
         cp_async16(dk + kScanThreads * 16, vb + (size_t)t * hrow);
@@ -301,8 +299,10 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     }
     cp_async_commit();
   };
-  issue(0);
-  issue(1);
+  if constexpr (!kWin) {
+    issue(0);
+    issue(1);
+  }
   // launched as a programmatic dependent of the plan: what follows reads its
   // outputs (the copies above read only the prompt)
   griddep_wait();
@@ -354,13 +354,13 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     if (a.weights != nullptr)  // the sign set as a bit: that of a negated NaN is unspecified
       a.weights[((size_t)chunk_id(t0, c, s) * L.Hkv + h) * kPrefillChunk + tid] =
           __uint_as_float((__float_as_uint(w) & 0x7fffffffu) | ((mine >> lane) & 1u) << 31);
-    if (lane == 0) { s_bal[warp] = mine; s_nbal[warp] = other; }
+    if (lane == 0) { s_bal[warp] = mine; s_bal[kPrefillChunk / 32 + warp] = other; }
   }
   __syncthreads();
   int nstart = 0, first = -1, next = -1;
 #pragma unroll
   for (int w = 0; w < kPrefillChunk / 32; ++w) {
-    const unsigned b = s_bal[w], nb = s_nbal[w];
+    const unsigned b = s_bal[w], nb = s_bal[kPrefillChunk / 32 + w];
     if (first < 0 && b) first = w * 32 + __ffs(b) - 1;
     if (next < 0 && nb) next = a1 + w * 32 + __ffs(nb) - 1;
     nstart += __popc(b);
@@ -372,6 +372,23 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     // to an earlier chunk's segment
     cp_async_wait<0>();
     return;
+  }
+  if constexpr (kWin) {
+    // Bit j of x: the token after the group's j-th opens a slot, or the prompt has
+    // ended. The j-th counts if one of bits j .. j + W - 1 is set (TPG + W <= 64).
+    const int q = g * TPG + 1, w0 = q >> 5;
+    unsigned long long x = (unsigned long long)s_bal[w0 + 1] << 32 | s_bal[w0];
+    if (q & 31) x = x >> (q & 31) | (unsigned long long)s_bal[w0 + 2] << (64 - (q & 31));
+    const int end = t1 - a0 - q;
+    if (end >= 0 && end < 64) x |= 1ull << end;
+    for (int n = 1; n < L.window;) {
+      const int d = min(n, L.window - n);
+      x |= x >> d;
+      n += d;
+    }
+    counts = (unsigned)x;
+    issue(0);
+    issue(1);
   }
   if (next < 0) {  // no opening in the next 128 tokens: search on (uniform)
     if (tid == 0) s_next = t1;
@@ -412,9 +429,10 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     xz += w;
   };
   auto add_row = [&](const uint4& kr, const uint4& vr, float w) { add_to(ak, av, zs, kr, vr, w); };
-  // The chunk's last segment runs on to `next`. Few rows there are its group's
-  // work; more are summed by all groups, 128 tokens at a time.
-  const bool long_tail = next - a1 > kLongTail && (!kWin || next - a1 < L.window);
+  // The chunk's last segment runs on to `next`, its rows from `tail` on are summed.
+  // Few are its group's work; more are summed by all groups, 128 tokens at a time.
+  const int tail = kWin ? max(a1, next - L.window) : a1;
+  const bool long_tail = next - tail > kLongTail;
   auto slot_ptr = [&](int slot) {
     const int page = s_page[slot / kPage - pfirst];
     return L.pages + (size_t)page * L.page_bytes + (size_t)(slot % kPage) * ROW + lr * 16;
@@ -439,18 +457,6 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     *reinterpret_cast<uint4*>(kdst + (size_t)kPage * ROW) = CK::pack(vn);
     if (lr == 0) L.z[(size_t)s_page[slot / kPage - pfirst] * kPage + slot % kPage] = zs;
   };
-  // window grouping: the sums of segment [tb, te), if it is longer than the window
-  auto window_sums = [&](int tb, int te) {
-    const int W = L.window;
-    if (te - tb <= W) return;
-    reset();
-#pragma unroll 1
-    for (int t = te - W; t < te; ++t) {
-      const uint4 kr = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)t * hrow));
-      const uint4 vr = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)t * hrow));
-      add_row(kr, vr, t < a1 && t >= a0 ? s_w[t - a0] : omega(t));
-    }
-  };
   auto group_bits = [&](int gg) {  // the opening tokens of group gg's range
     const unsigned b = s_bal[(gg * TPG) >> 5] >> ((gg * TPG) & 31);
     return TPG == 32 ? b : (b & ((1u << TPG) - 1u));
@@ -468,7 +474,6 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   }
   float hk[EPC], hv[EPC], hz = 0.f;  // the sums before the group's first opening
   bool open = false;                 // summing a segment that opened in this group
-  int opened = 0;                    // ... at this token (window grouping)
   reset();
   for (int b = 0; b < NB; ++b) {
     cp_async_wait<1>();  // copy group b has landed
@@ -478,7 +483,6 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
       if (t >= wb && t < g1) {
         if ((gbits >> (t - g0)) & 1u) {  // t opens a slot: the segment before it ends
           if (open) {
-            if constexpr (kWin) window_sums(opened, t);
             write_slot(slot);
           } else {
 #pragma unroll
@@ -487,9 +491,9 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
           }
           reset();
           open = true;
-          if constexpr (kWin) opened = t;
           ++slot;
         }
+        if (kWin && !(counts >> (t - g0) & 1u)) continue;
         const uint32_t sk = rk((b % 2) * kRingBatch + u);
         uint4 kr, vr;
         asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
@@ -528,27 +532,15 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
     }
     zs += from[2 * D];
   };
-  // Adds the rows tb, tb + step, ... below te, kAdd of them in flight. Two at a time
-  // in the exact kernel spill more than they hide (plan + scan of 32 x 2048 tokens at
-  // CR 32: 270 us with one, 281 with two; long ragged prompts 596 and 604), one at a
-  // time in the windowed one costs a 7B layer 331 us instead of 327.
-  constexpr int kAdd = kWin ? 2 : 1;
+  // Adds the rows tb, tb + step, ... below te, one at a time: two in flight spill more
+  // than they hide (plan + scan of 32 x 2048 tokens at CR 32: 270 us with one, 281 with
+  // two; long ragged prompts 596 and 604; windowed prompts 0-7 %).
   auto add_rows = [&](float* xk, float* xv, float& xz, int tb, int step, int te) {
 #pragma unroll 1
-    for (int t = tb; t < te; t += kAdd * step) {
-      uint4 kr[kAdd], vr[kAdd];
-      float w[kAdd];
-#pragma unroll
-      for (int u = 0; u < kAdd; ++u) {
-        if (t + u * step < te) {
-          kr[u] = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)(t + u * step) * hrow));
-          vr[u] = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)(t + u * step) * hrow));
-          w[u] = omega(t + u * step);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kAdd; ++u)
-        if (t + u * step < te) add_to(xk, xv, xz, kr[u], vr[u], w[u]);
+    for (int t = tb; t < te; t += step) {
+      const uint4 kr = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)t * hrow));
+      const uint4 vr = __ldg(reinterpret_cast<const uint4*>(vb + (size_t)t * hrow));
+      add_to(xk, xv, xz, kr, vr, omega(t));
     }
   };
   auto tail_sums = [&](int pb) {  // this group's rows among [pb, min(next, pb + 128))
@@ -559,7 +551,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
   };
   put(heads);
   if (long_tail) {
-    tail_sums(a1);
+    tail_sums(tail);
     put(tails);
   }
   __syncthreads();
@@ -587,7 +579,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
 #pragma unroll 1
       for (int i = 0; i < NG; ++i) add(tails + i * HS);
     } else {
-      add_rows(ak, av, zs, a1, 1, next);
+      add_rows(ak, av, zs, tail, 1, next);
     }
     return true;
   };
@@ -610,42 +602,37 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
       hz = zs;
     }
     slot = base - 1;
-    const int te = segment_end(-1);
-    if (kWin && te - t0 > L.window) {
-      window_sums(t0, te);
-    } else {
-      if constexpr (kWin) {
-        // the continued segment's tokens still inside the window
-        reset();
-        const int W = L.window;
-        const int parity = *reinterpret_cast<const volatile int*>(&L.ctl[a.layer * 4]);
-        const int n_old = L.seglen[((size_t)a.layer * 2 + parity) * L.NH + bh];
-        const int m = min(n_old, W - (te - t0));
-        const char* old = L.ring + ((size_t)a.layer * L.NH + bh) * W * 2 * ROW + lr * 16;
-        const float* old_w = L.ring_w + ((size_t)a.layer * L.NH + bh) * W;
+    if constexpr (kWin) {
+      // the continued segment's tokens still inside the window
+      reset();
+      const int W = L.window, te = segment_end(-1);
+      const int parity = *reinterpret_cast<const volatile int*>(&L.ctl[a.layer * 4]);
+      const int n_old = L.seglen[((size_t)a.layer * 2 + parity) * L.NH + bh];
+      const int m = min(n_old, W - (te - t0));
+      const char* old = L.ring + ((size_t)a.layer * L.NH + bh) * W * 2 * ROW + lr * 16;
+      const float* old_w = L.ring_w + ((size_t)a.layer * L.NH + bh) * W;
 #pragma unroll 2
-        for (int e = 0; e < m; ++e) {
-          const int pos = (n_old - 1 - e) % W;
-          add_row(*reinterpret_cast<const uint4*>(old + (size_t)pos * 2 * ROW),
-                  *reinterpret_cast<const uint4*>(old + (size_t)pos * 2 * ROW + ROW), old_w[pos]);
-        }
-      } else {
-        // the old slot's K z_old, V z_old and z_old start the sums
-        const char* kold = slot_ptr(slot);
-        float ko[EPC], vo[EPC];
-        CK::unpack(*reinterpret_cast<const uint4*>(kold), ko);
-        CK::unpack(*reinterpret_cast<const uint4*>(kold + (size_t)kPage * ROW), vo);
-        const float zo = L.z[(size_t)s_page[slot / kPage - pfirst] * kPage + slot % kPage];
-#pragma unroll
-        for (int e = 0; e < EPC; ++e) {
-          ak[e] = ko[e] * zo;
-          av[e] = vo[e] * zo;
-        }
-        zs = zo;
-        if (carry) put_carry(t0);  // the state the prompt's first token continues
+      for (int e = 0; e < m; ++e) {
+        const int pos = (n_old - 1 - e) % W;
+        add_row(*reinterpret_cast<const uint4*>(old + (size_t)pos * 2 * ROW),
+                *reinterpret_cast<const uint4*>(old + (size_t)pos * 2 * ROW + ROW), old_w[pos]);
       }
-      past = finish(-1);
+    } else {
+      // the old slot's K z_old, V z_old and z_old start the sums
+      const char* kold = slot_ptr(slot);
+      float ko[EPC], vo[EPC];
+      CK::unpack(*reinterpret_cast<const uint4*>(kold), ko);
+      CK::unpack(*reinterpret_cast<const uint4*>(kold + (size_t)kPage * ROW), vo);
+      const float zo = L.z[(size_t)s_page[slot / kPage - pfirst] * kPage + slot % kPage];
+#pragma unroll
+      for (int e = 0; e < EPC; ++e) {
+        ak[e] = ko[e] * zo;
+        av[e] = vo[e] * zo;
+      }
+      zs = zo;
+      if (carry) put_carry(t0);  // the state the prompt's first token continues
     }
+    past = finish(-1);
     if (nstart > 0) {
       write_slot(slot);
       past = false;
@@ -659,14 +646,7 @@ __global__ void __launch_bounds__(kScanThreads, 6) dmc_prefill_scan_kernel(const
       mine = true;  // the chunk's only segment: below
     }
   }
-  if (open) {
-    const int te = kWin ? segment_end(g) : 0;
-    if (kWin && te - opened > L.window) {
-      window_sums(opened, te);
-    } else {
-      past = finish(g);
-    }
-  }
+  if (open) past = finish(g);
   if constexpr (!kWin) {
     // a segment that runs on beyond the 128 tokens from a1
     for (int pb = a1 + kPrefillChunk; pb < next; pb += kPrefillChunk) {
