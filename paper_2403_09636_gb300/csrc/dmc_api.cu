@@ -18,7 +18,6 @@ cudaError_t prefill_launch(const Layout& L, int layer, int first_seq, int num_se
                            long long q_tok, long long q_head, const void* k, const void* v,
                            const int* cu, int total_tokens, int max_seqlen, float* carry,
                            float* weights, cudaStream_t stream);
-bool prefill_attn_supported(const Layout& L);
 cudaError_t prefill_attn_launch(const Layout& L, int layer, int first_seq, int num_seqs,
                                 const void* q, const void* k, const void* v, const int* cu,
                                 int total_tokens, int max_seqlen, const float* carry,
@@ -116,8 +115,10 @@ Offsets offsets(const dmc_cache_config* c) {
   o.pending_z = at; at = align_up(at + pend * 4);
   o.opens = at; at = align_up(at + (size_t)c->num_kv_heads * o.plan_stride * 16);
   o.plan = at; at = align_up(at + (size_t)c->num_kv_heads * o.plan_stride * 4);
-  o.carry = at; at = align_up(at + (size_t)o.plan_stride * c->num_kv_heads * (2 * c->head_dim + 1) * 4);
-  o.weights = at; at = align_up(at + (size_t)o.plan_stride * c->num_kv_heads * dmc::kPrefillChunk * 4);
+  const bool attends = dmc::prompt_attention(esize, c->head_dim, G, c->window);
+  const size_t attended = attends ? (size_t)o.plan_stride * c->num_kv_heads : 0;
+  o.carry = at; at = align_up(at + attended * (2 * c->head_dim + 1) * 4);
+  o.weights = at; at = align_up(at + attended * dmc::kPrefillChunk * 4);
   o.ring = at; at = align_up(at + (size_t)c->num_layers * NH * c->window * 2 * row);
   o.ring_w = at; at = align_up(at + (size_t)c->num_layers * NH * c->window * 4);
   o.total = at;
@@ -322,7 +323,7 @@ dmc_status dmc_prefill_attention(dmc_cache_t c, int32_t layer, int32_t first_seq
                                  cudaStream_t stream) {
   if (!c) return DMC_ERR_INVALID_ARG;
   const Layout& L = c->lay;
-  if (!dmc::prefill_attn_supported(L) || L.window != 0) return DMC_ERR_INVALID_ARG;
+  if (!dmc::prompt_attention(L.esize, L.D, L.G, L.window)) return DMC_ERR_INVALID_ARG;
   if (layer < 0 || layer >= L.L || first_seq < 0 || num_seqs < 0 || first_seq + num_seqs > L.B)
     return DMC_ERR_INVALID_ARG;
   if (total_tokens < 0 || total_tokens > L.max_prefill_tokens || max_seqlen < 0 ||

@@ -72,6 +72,11 @@ struct DecodePlan {
                        // the tensor-core kernel uses grid, smem
 };
 
+// Caches that prompt attention serves.
+inline bool prompt_attention(int esize, int head_dim, int group, int window) {
+  return esize == 2 && head_dim == 128 && (group == 1 || group == 2 || group == 4 || group == 8) && window == 0;
+}
+
 // ---------------------------------------------------------------- dtype helpers
 template <typename T> struct Elt;
 template <> struct Elt<float> {

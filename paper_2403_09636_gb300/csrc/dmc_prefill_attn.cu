@@ -1052,10 +1052,6 @@ dmc_prefill_attn_kernel(const PrefillAttnArgs a, const __grid_constant__ PaMaps 
   }
 }
 
-bool prefill_attn_supported(const Layout& L) {
-  return L.esize == 2 && L.D == kPaD && (L.G == 1 || L.G == 2 || L.G == 4 || L.G == 8);
-}
-
 // A 3-D bf16 tensor map: rows of 128 columns (box 64, 128-byte swizzle), `ny`
 // rows of stride `sy` bytes (box by), `nz` planes of stride `sz` bytes (box bz).
 static cudaError_t pa_map(CUtensorMap* map, const void* base, uint64_t ny, uint64_t sy, uint32_t by, uint64_t nz,
