@@ -260,11 +260,10 @@ class DmcCache:
         ids = t.as_tensor(head_ids, dtype=t.int32, device=self.device)
         n = ids.numel()
         D = self.cfg.head_dim
-        make = t.empty if n else t.zeros  # padded: every row is written
-        k = make((n, cap, D), dtype=self.dtype, device=self.device)
-        v = make((n, cap, D), dtype=self.dtype, device=self.device)
-        z = make((n, cap), dtype=t.float32, device=self.device)
-        ln = make(n, dtype=t.int32, device=self.device)
+        k = t.empty((n, cap, D), dtype=self.dtype, device=self.device)  # padded: every row is written
+        v = t.empty((n, cap, D), dtype=self.dtype, device=self.device)
+        z = t.empty((n, cap), dtype=t.float32, device=self.device)
+        ln = t.empty(n, dtype=t.int32, device=self.device)
         _check(dmc_cache_export_heads_padded(self.handle, layer, n, ids.data_ptr(), cap,
                                              k.data_ptr(), v.data_ptr(), z.data_ptr(),
                                              ln.data_ptr(), self._s(stream)),

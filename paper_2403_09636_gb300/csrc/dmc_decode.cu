@@ -31,9 +31,9 @@
 // Programmatic dependent launch: everything before griddep_wait() reads only
 // this layer's cache state (lengths, page table, pages), never q, k, v or
 // anything a preceding kernel of another layer writes, so it may overlap the
-// tail of the previous kernel on the stream. The host does not use the
-// attribute when the previous decode launch of the cache was for the same
-// layer. (Using it there too, with the wait at the kernel's very start, saves the
+// tail of the previous kernel on the stream. The host uses the attribute only
+// behind the cache's decode of other layers on the same stream (dmc_overlap.h).
+// (Using it behind the same layer too, with the wait at the kernel's very start, saves the
 // GPU 0.7 us per launch of a one-layer cache and costs the host 2.)
 #include <math.h>
 
@@ -168,7 +168,7 @@ __device__ __noinline__ void combine_partials(const float* partials, int wf, int
       if (i0 + c0 > 0) load(i0 + c0);
 #pragma unroll
       for (int r = 0; r < NR; ++r) {
-        const int c = c0 + 4 * r + cg;  // < 32
+        const int c = c0 + 4 * r + cg;  // may pass 31 (the shuffle wraps): dropped below
         const float wv = __shfl_sync(0xffffffffu, w, c);
         if (c < n32) {
 #pragma unroll
@@ -291,7 +291,8 @@ dmc_decode_kernel(const DecodeArgs a) {
   // each, spread over the blocks so that every SM takes part. Such a launch is
   // all latency: cutting the list over every warp left empty ranges between
   // the parts, which each finish and merge had to step over (7B shape, batch 1,
-  // ~550 units on 1824 warps: 45.2 us per launch, 13.1 with one unit each). If
+  // ~550 units on the 1824 warps of that time: 45.2 us per launch, 13.1 with one
+  // unit each, 10.2 now). If
   // the first half of the blocks can take them all, the others leave at once, and
   // the next launch's blocks start its prologue in their place.
   const bool few = Utot < (long long)gridDim.x * NWARP;
