@@ -88,6 +88,11 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&h);
 }
+// What pack_bf16x2 rounded off, as bf16 in turn: the pair's sum holds 16 bits or more of
+// each value.
+__device__ __forceinline__ uint32_t pack_rest(float lo, float hi, uint32_t packed) {
+  return pack_bf16x2(lo - __uint_as_float(packed << 16), hi - __uint_as_float(packed & 0xffff0000u));
+}
 
 // Workers of a layer of U units over nh heads, on a grid of `warps` warps. A
 // worker streams a page unit in about kUnitCost times what the merge of a split
@@ -425,6 +430,7 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
       const float2 c2 = make_float2(__shfl_sync(0xffffffffu, corr, 8 * t), __shfl_sync(0xffffffffu, corr, 8 * t + 4));
       const uint32_t p00 = pack_bf16x2(p[0], p[1]), p01 = pack_bf16x2(p[2], p[3]);
       const uint32_t p10 = pack_bf16x2(p[4], p[5]), p11 = pack_bf16x2(p[6], p[7]);
+      const uint32_t r00 = pack_rest(p[0], p[1], p00), r01 = pack_rest(p[2], p[3], p01);
       const uint32_t vtile = tile + kTile * ROW;
 #pragma unroll
       for (int mt = 0; mt < KT; ++mt) {
@@ -436,13 +442,16 @@ __global__ void __launch_bounds__(kGThreads, 1) dmc_decode_gqa_kernel(const GqaA
         uint32_t a0, a1, a2, a3;
         ldmatrix_x4_trans(vtile + swz(srow, mt * 2 + (mi & 1), ROW), a0, a1, a2, a3);
         mma_bf16_16816(o[mt], a0, a1, a2, a3, p00, p01);
+        mma_bf16_16816(o[mt], a0, a1, a2, a3, r00, r01);
       }
       if (two) {
+        const uint32_t r10 = pack_rest(p[4], p[5], p10), r11 = pack_rest(p[6], p[7], p11);
 #pragma unroll
         for (int mt = 0; mt < KT; ++mt) {
           uint32_t a0, a1, a2, a3;
           ldmatrix_x4_trans(vtile + kHalf * ROW + swz(srow, mt * 2 + (mi & 1), ROW), a0, a1, a2, a3);
           mma_bf16_16816(o[mt], a0, a1, a2, a3, p10, p11);
+          mma_bf16_16816(o[mt], a0, a1, a2, a3, r10, r11);
         }
       }
     };
