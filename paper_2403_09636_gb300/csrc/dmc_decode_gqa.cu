@@ -13,7 +13,14 @@
 //
 // The score fragment (row = query, cols = 2 slots) is exactly the B operand
 // layout of the second product, so P never leaves registers and the output
-// accumulator O^T has no padded rows. K and V move in tiles of 32 slots (a
+// accumulator O^T has no padded rows. P enters it twice, rounded to bf16 and what that
+// rounding left, with the V fragments of one load: rounded once, the outputs' error
+// depended on how many slots were the maximum of a step (their weight is exactly one),
+// so that longer steps and fewer workers raised it by 1-4 % (rms against 64 bits, of
+// outputs that round to bf16 themselves, 8 x 2000 tokens at 2x, G = 8: relative 2.15e-3
+// with 16-slot steps, 2.18e-3 with 32, 1.79e-3 so). It adds 16 products to a page's 48
+// (70B batch 64: 89.7 -> 92.6 us per launch; interleaved or in a pass of its own the
+// same). K and V move in tiles of 32 slots (a
 // page): each lane cp.asyncs 16-byte chunks into a per-warp ring in shared
 // memory, chunks XOR-swizzled by row so that ldmatrix (and ldmatrix.trans for
 // V) reads without bank conflicts; rows past the head's length are
@@ -37,7 +44,7 @@ constexpr int kGThreads = kGWarps * 32;
 // Tiles per warp ring (all but one in flight): a cache with so many heads that the
 // unit prefixes leave no room for three takes two. A page per softmax step halves
 // the shuffles, exponentials of the running maximum and accumulator rescales of the
-// 16-slot tiles before (70B batch 64: 93.8 -> 90.2 us per launch, 89.7 now). Warps x ring,
+// 16-slot tiles before (70B batch 64: 93.8 -> 90.2 us per launch). Warps x ring,
 // one block per SM: 4 x 3 90.2, 3 x 4 113.1, 5 x 2 91.3, 6 x 2 91.8.
 constexpr int kGRing = 3;
 constexpr int kGRingMany = 2;
