@@ -52,18 +52,19 @@ namespace dmc {
 // with HBM: us per launch against 6 warps with one row, 7B batch 32 49.1 (51.1),
 // head_dim 64 34.5 (38.5), window 12 50.6 (53.4). Over several layers six (against 8
 // with one row; five are as fast on long heads, but 2560 heads of 24 slots took 25.6 us
-// a layer with five, 17.6 with six and 21.5 with the eight before): 4 layers of mixed
-// ratios 5.99 ms a generation with six, 5.97 with five.
+// a layer with five, 17.6 with six and 21.5 with the eight before).
 constexpr int kWarpsOne = kDecodeWarpsPerBlock;
 constexpr int kWarpsWalk = kDecodeWalkWarpsPerBlock;
 constexpr int kRows = 8;        // slot rows per piece: rows grp and grp + 4 of it are an 8-lane group's
 // Pieces per warp ring (all but one in flight). Measured with 4 / 5 / 6 / 8 warps per
 // block, two blocks per SM, us per launch of the 7B shape at batch 32: ring 3 49.9 /
-// 49.5 / 49.7 / 60.7, ring 4 49.0 / 50.7 / 51.2 / -; over four layers of mixed ratios
-// per layer-step (a whole generation, ms): ring 3 - / 5.97 / 5.99 / 6.03, ring 4 6.06
-// / 6.16 / - / 6.17. Rows of 512 bytes keep ring 3, so that two blocks still fit.
+// 49.5 / 49.7 / 60.7, ring 4 49.0 / 50.7 / 51.2 / -. Six warps over rows of 256 bytes or
+// more take two: ~1000 slots of 10,240 heads 810 us per launch with three, 767 with two
+// (4 warps 795), one launch for several layers 812 and 767; 24 slots of 4096 heads 23.8
+// and 24.3; rows of 128 bytes 107 and 121 with ~600 slots of 4096 heads. Rows of 512
+// bytes keep ring 3 with four warps, so that two blocks still fit.
 template <int ROW, int NWARP>
-constexpr int kRing = NWARP == kWarpsOne && ROW < 512 ? 4 : 3;
+constexpr int kRing = NWARP == kWarpsOne ? (ROW < 512 ? 4 : 3) : ROW < 256 ? 3 : 2;
 constexpr int kWindow = 64;     // page units per warp window (page id + rows to copy)
 constexpr int kHeadWindow = 32; // heads whose gates a warp holds in its lanes
 constexpr int kMaxDecodeBlocks = 512;
