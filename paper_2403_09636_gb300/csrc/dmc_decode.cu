@@ -52,16 +52,16 @@ namespace dmc {
 // with HBM: us per launch against 6 warps with one row, 7B batch 32 49.1 (51.1),
 // head_dim 64 34.5 (38.5), window 12 50.6 (53.4). Over several layers six (against 8
 // with one row; five are as fast on long heads, but 2560 heads of 24 slots took 25.6 us
-// a layer with five, 17.6 with six and 21.5 with the eight before).
+// a layer with five, 17.8 with six and 21.5 with the eight before).
 constexpr int kWarpsOne = kDecodeWarpsPerBlock;
 constexpr int kWarpsWalk = kDecodeWalkWarpsPerBlock;
 constexpr int kRows = 8;        // slot rows per piece: rows grp and grp + 4 of it are an 8-lane group's
 // Pieces per warp ring (all but one in flight). Measured with 4 / 5 / 6 / 8 warps per
 // block, two blocks per SM, us per launch of the 7B shape at batch 32: ring 3 49.9 /
 // 49.5 / 49.7 / 60.7, ring 4 49.0 / 50.7 / 51.2 / -. Six warps over rows of 256 bytes or
-// more take two: ~1000 slots of 10,240 heads 810 us per launch with three, 767 with two
+// more take two: ~1000 slots of 10,240 heads 810 us per launch with three, 768 with two
 // (4 warps 795), one launch for several layers 812 and 767; 24 slots of 4096 heads 23.8
-// and 24.3; rows of 128 bytes 107 and 121 with ~600 slots of 4096 heads. Rows of 512
+// and 23.9; rows of 128 bytes 107 and 121 with ~600 slots of 4096 heads. Rows of 512
 // bytes keep ring 3 with four warps, so that two blocks still fit.
 template <int ROW, int NWARP>
 constexpr int kRing = NWARP == kWarpsOne ? (ROW < 512 ? 4 : 3) : ROW < 256 ? 3 : 2;
@@ -216,7 +216,7 @@ __device__ __noinline__ void combine_partials(const float* partials, int wf, int
 // into their pages. In 16-byte pieces, kBatch per thread in flight: it is the launch's
 // tail, on one block. (A thread per head, one piece after the other, took a launch
 // 13 us for every blockDim.x heads: fp32, 4 queries per KV head, d 128, 24 tokens, us
-// per launch at batch 16 / 32 / 48 / 64: 29 / 52 / 72 / 95 so, 21 / 37 / 50 / 67 now.)
+// per launch at batch 16 / 32 / 48 / 64: 29 / 52 / 72 / 95 so, 21 / 38 / 52 / 58 now.)
 template <int ROW>
 __device__ __noinline__ void write_pending(char* pages, float* z, int nh, const char* pending, const int* pending_at,
                                            const float* pending_z) {
@@ -878,9 +878,9 @@ static cudaError_t setup_decode(int nvh, DecodePlan* plan) {
   if (e == cudaErrorInvalidConfiguration) e = cudaSuccess;
   // With more than 3 heads for every 2 warps a layer of short heads is a chain of owner
   // updates on each warp, and takes the shape with more warps (bf16 d 128, 24 slots, us
-  // per launch with 4 / 6 warps: 1536 heads 16.2 / 17.8, 1792 16.6 / 16.4, 2048 21.9 /
-  // 16.9, 4096 41.5 / 25.1, 8192 73.4 / 40.8; of ~520 slots: 1024 heads 48.8 / 49.5,
-  // 1536 69.5 / 70.3, 2048 90.9 / 90.6). Lengths are not known on the host.
+  // per launch with 4 / 6 warps: 1536 heads 16.2 / 17.8, 1792 16.6 / 16.4, 2048 21.7 /
+  // 15.9, 4096 41.3 / 23.9, 8192 73.4 / 38.6; of ~520 slots: 1024 heads 48.8 / 49.5,
+  // 1536 69.5 / 70.3, 2048 90.9 / 89.3). Lengths are not known on the host.
   if (plan->grid_walk > 0 && (long long)nvh * 2 > (long long)plan->grid * kWarpsOne * 3) {
     plan->grid = plan->grid_walk;
     plan->smem = plan->smem_walk;

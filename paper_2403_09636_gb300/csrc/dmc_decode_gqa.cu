@@ -19,7 +19,7 @@
 // so that longer steps and fewer workers raised it by 1-4 % (rms against 64 bits, of
 // outputs that round to bf16 themselves, 8 x 2000 tokens at 2x, G = 8: relative 2.15e-3
 // with 16-slot steps, 2.18e-3 with 32, 1.79e-3 so). It adds 16 products to a page's 48
-// (70B batch 64: 89.7 -> 92.6 us per launch; interleaved or in a pass of its own the
+// (70B batch 64: 89.7 -> 92.2 us per launch; interleaved or in a pass of its own the
 // same). K and V move in tiles of 32 slots (a
 // page): each lane cp.asyncs 16-byte chunks into a per-warp ring in shared
 // memory, chunks XOR-swizzled by row so that ldmatrix (and ldmatrix.trans for
